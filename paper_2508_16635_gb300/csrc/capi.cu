@@ -26,7 +26,7 @@
 #include "krylov_split.cuh"
 #include "chain_df.cuh"
 #include "chain_cr.cuh"
-#include "products_lin.cuh"
+#include "products_sym.cuh"
 #include "radial_rhs_f32.cuh"
 #include "cr_factor_gpu.cuh"
 #include "factor_gpu.cuh"
@@ -109,7 +109,6 @@ struct rsc_ctx {
   void *SR = nullptr, *FC = nullptr, *FCU = nullptr, *FA = nullptr, *AR = nullptr;
   void* AR0 = nullptr;   // analysed products of x^n during a second-order step
   void* UG = nullptr;    // grid values of the cached base state, [9][Nd][nlat][nphi]
-  int ug_prec = 0;       // precision UG holds for the current FCU: 0 none, 1 FP64, 2 FP32
   double2* rhs = nullptr;
   double2* mid = nullptr;   // chain sweep staging, [2 nm][3][Nr]
   double* xtmp = nullptr;
@@ -487,12 +486,21 @@ int radial_fixed(const Dims& d) {
   return (d.Nr == 64 && d.Nd == 96) ? 1 : (d.Nr == 96 && d.Nd == 144) ? 2 : 0;
 }
 
+template <typename R, int J>
+rsc_status products_attributes(rsc_ctx* ctx, int bytes) {
+  const void* fns[] = {
+      (const void*)k_products<R, kProdStep, true, J>, (const void*)k_products<R, kProdStep, false, J>,
+      (const void*)k_products<R, kProdLin, true, J>, (const void*)k_products<R, kProdLin, false, J>,
+      (const void*)k_products<R, kProdBase, true, J>, (const void*)k_products<R, kProdBase, false, J>};
+  for (const void* fn : fns) CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  return RSC_OK;
+}
+
 rsc_status set_smem_limits(rsc_ctx* ctx) {
   const int big = 200 * 1024;
-  CK(cudaFuncSetAttribute(k_products<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  CK(cudaFuncSetAttribute(k_products<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  CK(cudaFuncSetAttribute(k_products<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  CK(cudaFuncSetAttribute(k_products<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  CKS((products_attributes<double, 1>(ctx, big)));
+  CKS((products_attributes<float, 1>(ctx, big)));
+  CKS((products_attributes<float, 2>(ctx, big)));
   CK(cudaFuncSetAttribute(k_radial<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   CK(cudaFuncSetAttribute(k_radial<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   {
@@ -1041,7 +1049,8 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
   return RSC_OK;
 }
 
-// Shared memory of the DFT + products kernel for `wpb` warps per block.
+// Bound on the `products_warps` field of rsc_tuning (the shared memory of `wpb` warps with all
+// twiddles staged); the shape of k_products itself follows from the sizes (prod_shape).
 template <typename R>
 size_t products_smem(const Dims& d, bool lin, int wpb) {
   using V = typename C2<R>::T;
@@ -1065,6 +1074,33 @@ size_t rhs_smem(const Dims& d, int ppb) {
                         4 * (size_t)d.Nd * sizeof(V));
 }
 
+// k_products on the coefficients `fc`, mode kProdStep, kProdLin or kProdBase.
+template <typename R>
+void launch_products(rsc_ctx* ctx, int mode, const ProdShape& ps, const void* fc) {
+  using V = typename C2<R>::T;
+  const Dims& d = ctx->d;
+  const DevGeom g = ctx->geom();
+  const DevLegendre<R> T = leg<R>(ctx).view();
+  const dim3 grid(d.Nd, (d.nlat + ps.LT - 1) / ps.LT);
+  const V* c = reinterpret_cast<const V*>(fc);
+  V* fa = reinterpret_cast<V*>(ctx->FA);
+  R* ug = reinterpret_cast<R*>(ctx->UG);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, ps.LT * ps.S, ps.smem, ctx->s>>>(g, T, (R)ctx->p.Ek, c, fa, ug, ps.LT, ps.S, ps.Q);
+  };
+  auto pick = [&](auto even, auto quads) {
+    constexpr bool E = decltype(even)::value;
+    constexpr int J = decltype(quads)::value;
+    if (mode == kProdStep) go(k_products<R, kProdStep, E, J>);
+    else if (mode == kProdLin) go(k_products<R, kProdLin, E, J>);
+    else go(k_products<R, kProdBase, E, J>);
+  };
+  using one = std::integral_constant<int, 1>;
+  using two = std::integral_constant<int, sizeof(R) == 4 ? 2 : 1>;
+  if (d.nphi % 2 == 0) ps.J == 2 ? pick(std::true_type{}, two{}) : pick(std::true_type{}, one{});
+  else ps.J == 2 ? pick(std::false_type{}, two{}) : pick(std::false_type{}, one{});
+}
+
 template <typename R>
 rsc_status stage_products_analysis(rsc_ctx* ctx, bool lin) {
   using V = typename C2<R>::T;
@@ -1072,48 +1108,15 @@ rsc_status stage_products_analysis(rsc_ctx* ctx, bool lin) {
   const DevGeom g = ctx->geom();
   const LegDev<R>& L = leg<R>(ctx);
   const int K1 = d.K + 1;
-  const int NF = lin ? 18 : 9;
-  int WPB = ctx->wpb[sizeof(R) == 4 ? 1 : 0] > 0 ? ctx->wpb[sizeof(R) == 4 ? 1 : 0] : 8;
-  auto smem_for = [&](int wpb) { return products_smem<R>(d, lin, wpb); };
-  while (WPB > 1 && smem_for(WPB) > 190 * 1024) WPB /= 2;
-  const size_t smem = smem_for(WPB);
-  const int LPW = ctx->lpw[sizeof(R) == 4 ? 1 : 0];
-  dim3 grid(d.Nd, (d.nlat + WPB * LPW - 1) / (WPB * LPW));
   const double npts = (double)d.Nd * d.nlat * d.nphi;
-  // Jacobian actions read the base state's grid values (k_base_grid) when they are cached
-  const bool ug = lin && ctx->ug_prec == (sizeof(R) == 4 ? 2 : 1);
-  const int nft = ug ? 9 : NF;   // fields transformed
+  // inverse DFT 9 fields, forward DFT 4 products; Jacobian actions also read the base state's
+  // grid values (kProdBase, once per base state)
   {
+  const ProdShape ps = prod_shape<R>(K1, d.nphi, d.nlat, d.Nd, false);
   KSpan sp(ctx, RSC_K_PRODUCTS,
-           (double)(nft + 4) * d.Nd * K1 * d.nlat * sizeof(V) + (ug ? 9.0 * npts * sizeof(R) : 0.0),
-           npts * (4.0 * nft * d.K + (lin ? 60.0 : 30.0) + 16.0 * K1));
-  bool done = false;
-  if constexpr (sizeof(R) == 4) {
-    // Jacobian actions on the small transforms of the wave workloads
-    // (the kernel's gather offsets are 32-bit: 9 Nd (K + 1) nlat coefficients per field set)
-    if (lin && ug && d.nphi <= 32 && K1 <= 12 && WPB <= kPlMaxWarps &&
-        9.0 * d.Nd * K1 * d.nlat < 2147483647.0) {
-      const float2* fc = reinterpret_cast<const float2*>(ctx->FC);
-      float2* fa = reinterpret_cast<float2*>(ctx->FA);
-      const float* ugp = reinterpret_cast<const float*>(ctx->UG);
-      // (nphi >= 3 K + 1, so nphi <= 32 keeps K + 1 <= 11)
-      if (K1 <= 8)
-        k_products_lin<8><<<grid, 32 * WPB, 0, ctx->s>>>(g, L.view(), (float)ctx->p.Ek, fc, fa, LPW, ugp);
-      else
-        k_products_lin<12><<<grid, 32 * WPB, 0, ctx->s>>>(g, L.view(), (float)ctx->p.Ek, fc, fa, LPW, ugp);
-      done = true;
-    }
-  }
-  if (done) {
-  } else if (lin)
-    k_products<R, true><<<grid, 32 * WPB, smem, ctx->s>>>(
-        g, L.view(), (R)ctx->p.Ek, reinterpret_cast<const V*>(ctx->FC),
-        reinterpret_cast<const V*>(ctx->FCU), reinterpret_cast<V*>(ctx->FA), LPW,
-        ug ? reinterpret_cast<const R*>(ctx->UG) : nullptr);
-  else
-    k_products<R, false><<<grid, 32 * WPB, smem, ctx->s>>>(
-        g, L.view(), (R)ctx->p.Ek, reinterpret_cast<const V*>(ctx->FC), nullptr,
-        reinterpret_cast<V*>(ctx->FA), LPW, nullptr);
+           13.0 * d.Nd * K1 * d.nlat * sizeof(V) + (lin ? 9.0 * npts * sizeof(R) : 0.0),
+           npts * (36.0 * d.K + (lin ? 60.0 : 30.0) + 16.0 * K1));
+  launch_products<R>(ctx, lin ? kProdLin : kProdStep, ps, ctx->FC);
   CK(cudaGetLastError());
   }
   {
@@ -1773,22 +1776,17 @@ template <typename R>
 rsc_status base_grid(rsc_ctx* ctx) {
   using V = typename C2<R>::T;
   const Dims& d = ctx->d;
-  const int K1 = d.K + 1, WPB = 8;
+  const int K1 = d.K + 1;
   KSpan sp(ctx, RSC_K_PRODUCTS,
            9.0 * d.Nd * K1 * d.nlat * sizeof(V) + 9.0 * d.Nd * d.nlat * d.nphi * sizeof(R),
            (double)d.Nd * d.nlat * d.nphi * 36.0 * K1);
-  k_base_grid<R><<<dim3(d.Nd, (d.nlat + WPB - 1) / WPB), 32 * WPB,
-                   (size_t)WPB * 9 * K1 * sizeof(V), ctx->s>>>(
-      ctx->geom(), leg<R>(ctx).view(), reinterpret_cast<const V*>(ctx->FCU),
-      reinterpret_cast<R*>(ctx->UG));
+  launch_products<R>(ctx, kProdBase, prod_shape<R>(K1, d.nphi, d.nlat, d.Nd, true), ctx->FCU);
   CK(cudaGetLastError());
-  ctx->ug_prec = sizeof(R) == 4 ? 2 : 1;
   return RSC_OK;
 }
 
 // Base-state grid coefficients (and grid values) for Jacobian actions.
 rsc_status cache_base(rsc_ctx* ctx, const double* U, bool fp32) {
-  ctx->ug_prec = 0;
   if (fp32) {
     CKS(stage_synth<float>(ctx, U, ctx->FCU));
     return base_grid<float>(ctx);
@@ -2278,27 +2276,11 @@ rsc_status tune_precision(rsc_ctx* ctx, rsc_tuning& t, cudaEvent_t e0, cudaEvent
     return st == RSC_OK ? ms / 3.0 : 1e30;
   };
   CKS(stage_synth<R>(ctx, ctx->rtmp, ctx->FC));
-  ctx->ug_prec = 0;
   CKS(stage_synth<R>(ctx, ctx->rtmp, ctx->FCU));
   CKS(base_grid<R>(ctx));
   auto pa = [&] { return stage_products_analysis<R>(ctx, true); };
-  // products: warps per block x latitudes per warp
-  double best = 1e30;
-  int bw = t.products_warps[p], bl = t.products_lats[p];
-  for (int w : {1, 2, 4, 8}) {
-    if (products_smem<R>(d, true, w) > 190 * 1024) continue;
-    for (int lp : {1, 2, 4, 8}) {
-      ctx->wpb[p] = w;
-      ctx->lpw[p] = lp;
-      const double ms = timeit(pa);
-      CKS(st);
-      if (ms < best) { best = ms; bw = w; bl = lp; }
-    }
-  }
-  ctx->wpb[p] = t.products_warps[p] = bw;
-  ctx->lpw[p] = t.products_lats[p] = bl;
   // analysis: radii per block x latitudes per staged table chunk
-  best = 1e30;
+  double best = 1e30;
   int br = t.analysis_radii[p], bc = t.analysis_chunk[p];
   const int rmax = radii_limit((const void*)k_analysis<R>, round32(d.L + 1));
   for (int r = 1; r <= rmax; r *= 2) {

@@ -262,164 +262,6 @@ __global__ void k_synth(DevGeom g, DevLegendre<R> T, const typename C2<R>::T* __
 }
 
 // ---------------------------------------------------------------------------
-// a3-a5: inverse DFT, products, forward DFT.  grid = (Nd, ceil(nlat / (WPB LPW))),
-// block = 32 x WPB: warp w handles latitudes th0 + w + WPB r, r < LPW.  Inverse DFT: lane j
-// sums the (K+1) coefficients of each field at its longitudes (coefficients
-// are warp broadcasts, twiddles [a][j] are bank-conflict free).  Forward DFT:
-// lane a sums its wavenumber over the nphi longitudes (twiddles stored [j][a]).
-// LIN = false: F = Ek U x omega, N = U.grad T from FC.
-// LIN = true : F = Ek (U x omega_u + u x omega_U), N = U.grad tau + u.grad T
-//              with U from FCU and u from FC; when UG is given, U's grid values are read
-//              from it (k_base_grid, once per base state) instead of transformed again.
-template <typename R, bool LIN>
-__global__ void k_products(DevGeom g, DevLegendre<R> T, R Ek,
-                           const typename C2<R>::T* __restrict__ FC,
-                           const typename C2<R>::T* __restrict__ FCU,
-                           typename C2<R>::T* __restrict__ FA, int LPW,
-                           const R* __restrict__ UG) {
-  using V = typename C2<R>::T;
-  constexpr int NF = LIN ? 18 : 9;
-  extern __shared__ unsigned char sh_raw[];
-  const int K1 = g.K + 1, nphi = g.nphi, nlat = g.nlat, Nd = g.Nd;
-  const int WPB = blockDim.x >> 5;
-  V* coef = reinterpret_cast<V*>(sh_raw);                 // [WPB][NF][K1]
-  R* twc = reinterpret_cast<R*>(coef + WPB * NF * K1);    // [K1][nphi] (x2 for a > 0)
-  R* tws = twc + K1 * nphi;
-  R* twcT = tws + K1 * nphi;                              // [nphi][K1] / nphi
-  R* twsT = twcT + K1 * nphi;
-  R* prod = twsT + K1 * nphi;                             // [WPB][4][nphi + 1]
-  const int i = blockIdx.x;
-  const R inv = (R)1 / (R)nphi;
-  for (int idx = threadIdx.x; idx < K1 * nphi; idx += blockDim.x) {
-    const int a = idx / nphi, j = idx - a * nphi;
-    const R f = a ? (R)2 : (R)1;
-    const R c = T.twc[idx], sn = T.tws[idx];
-    twc[idx] = f * c;
-    tws[idx] = f * sn;
-    twcT[j * K1 + a] = c * inv;
-    twsT[j * K1 + a] = sn * inv;
-  }
-  __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  V* cw = coef + w * NF * K1;
-  const int pst = nphi + 1;   // padded row: the four products of one j sit in four banks
-  R* pw = prod + w * 4 * pst;
-  // warp w takes latitudes th0 + w, th0 + w + WPB, ... (LPW of them): the twiddles staged
-  // above serve all of them
-  const int th0 = blockIdx.y * WPB * LPW;
-  for (int rep = 0; rep < LPW; ++rep) {
-    const int th = th0 + w + WPB * rep;
-    if (th >= nlat) break;
-    const bool cached = LIN && UG != nullptr;
-    const int nfl = cached ? 9 : NF;   // fields transformed here
-    __syncwarp();
-    for (int idx = lane; idx < nfl * K1; idx += 32) {
-      const int a = idx % K1;
-      const int f = idx / K1;
-      const V* src = (f < 9) ? FC : FCU;
-      const int ff = (f < 9) ? f : f - 9;
-      V v = src[(((long)ff * Nd + i) * K1 + a) * nlat + th];
-      if (a == 0) v.y = 0;                // the m = 0 coefficient enters with its real part
-      cw[f * K1 + a] = v;
-    }
-    __syncwarp();
-    for (int j = lane; j < nphi; j += 32) {
-      R val[NF];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) val[f] = 0;
-      for (int a = 0; a < K1; ++a) {
-        const R c = twc[a * nphi + j], sn = tws[a * nphi + j];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          if (f < 9 || !cached) {
-            const V cf = cw[f * K1 + a];
-            val[f] += cf.x * c - cf.y * sn;
-          }
-        }
-      }
-      if (cached) {
-#pragma unroll
-        for (int f = 0; f < 9; ++f) val[(f + 9) % NF] = UG[(((long)f * Nd + i) * nlat + th) * nphi + j];
-      }
-      R Fr, Ft, Fp, N;
-      if (!LIN) {
-        // val: 0 ur 1 ut 2 up 3 wr 4 wt 5 wp 6 Tr 7 Tt 8 Tp
-        Fr = Ek * (val[1] * val[5] - val[2] * val[4]);
-        Ft = Ek * (val[2] * val[3] - val[0] * val[5]);
-        Fp = Ek * (val[0] * val[4] - val[1] * val[3]);
-        N = val[0] * val[6] + val[1] * val[7] + val[2] * val[8];
-      } else {
-        const R* u = val;      // perturbation
-        const R* U = val + 9;  // base state
-        Fr = Ek * ((U[1] * u[5] - U[2] * u[4]) + (u[1] * U[5] - u[2] * U[4]));
-        Ft = Ek * ((U[2] * u[3] - U[0] * u[5]) + (u[2] * U[3] - u[0] * U[5]));
-        Fp = Ek * ((U[0] * u[4] - U[1] * u[3]) + (u[0] * U[4] - u[1] * U[3]));
-        N = U[0] * u[6] + U[1] * u[7] + U[2] * u[8] + u[0] * U[6] + u[1] * U[7] + u[2] * U[8];
-      }
-      pw[0 * pst + j] = Fr;
-      pw[1 * pst + j] = Ft;
-      pw[2 * pst + j] = Fp;
-      pw[3 * pst + j] = N;
-    }
-    __syncwarp();
-    // forward DFT: one (product q, wavenumber a) output per lane, 4 (K + 1) outputs per
-    // latitude (a lane per wavenumber left 32 - (K + 1) lanes idle)
-    for (int t = lane; t < 4 * K1; t += 32) {
-      const int q = t / K1, a = t - q * K1;
-      const R* pq = pw + q * pst;
-      R sr = 0, si = 0;
-      for (int j = 0; j < nphi; ++j) {
-        const R v = pq[j];
-        sr += v * twcT[j * K1 + a];
-        si -= v * twsT[j * K1 + a];
-      }
-      FA[(((long)q * Nd + i) * K1 + a) * nlat + th] = mk<R>(sr, si);
-    }
-  }
-}
-
-// The base state's nine grid fields UG[f][i][th][j] (f: u_r, u_th, u_ph, w_r, w_th, w_ph,
-// T_r, T_th, T_ph) from its Fourier coefficients FCU, with the inverse DFT of k_products;
-// computed once per base state so that every Jacobian action transforms only the
-// perturbation.  grid = (Nd, ceil(nlat / WPB)), block = 32 WPB (a warp per latitude),
-// dynamic shared memory WPB 9 (K+1) complex.
-template <typename R>
-__global__ void k_base_grid(DevGeom g, DevLegendre<R> T, const typename C2<R>::T* __restrict__ FCU,
-                            R* __restrict__ UG) {
-  using V = typename C2<R>::T;
-  extern __shared__ unsigned char sh_raw[];
-  const int K1 = g.K + 1, nphi = g.nphi, nlat = g.nlat, Nd = g.Nd;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  V* cw = reinterpret_cast<V*>(sh_raw) + w * 9 * K1;
-  const int i = blockIdx.x;
-  const int th = blockIdx.y * (blockDim.x >> 5) + w;
-  if (th >= nlat) return;
-  for (int idx = lane; idx < 9 * K1; idx += 32) {
-    const int a = idx % K1, f = idx / K1;
-    V v = FCU[(((long)f * Nd + i) * K1 + a) * nlat + th];
-    if (a == 0) v.y = 0;
-    cw[f * K1 + a] = v;
-  }
-  __syncwarp();
-  for (int j = lane; j < nphi; j += 32) {
-    R val[9];
-#pragma unroll
-    for (int f = 0; f < 9; ++f) val[f] = 0;
-    for (int a = 0; a < K1; ++a) {
-      const R fa = a ? (R)2 : (R)1;
-      const R c = fa * T.twc[a * nphi + j], sn = fa * T.tws[a * nphi + j];
-#pragma unroll
-      for (int f = 0; f < 9; ++f) {
-        const V cf = cw[f * K1 + a];
-        val[f] += cf.x * c - cf.y * sn;
-      }
-    }
-#pragma unroll
-    for (int f = 0; f < 9; ++f) UG[(((long)f * Nd + i) * nlat + th) * nphi + j] = val[f];
-  }
-}
-
-// ---------------------------------------------------------------------------
 // a6: Legendre analysis.  grid = (nm, ceil(Nd / blockDim.y)), block =
 // (>= L + 1, multiple of 32) x RT radii; the Legendre tables are staged TC latitudes at a
 // time (dynamic shared memory RT 8 nlat/2 sizeof(V) + TC 3 (L + 1) sizeof(R)).
