@@ -46,3 +46,38 @@ def test_products_longitude_counts(torch, L, Ms, precision):
                              200.0).cpu().numpy()
     assert max(_errors(s, got, s.jvp(x, 0.4, J, u, 200.0))) < (1e-11 if precision == "fp64" else 1e-5)
     gpu.close()
+
+
+# FP64 Legendre transforms on digit slices: degrees per parity class 16 and 17 (one and two 16-term
+# steps), m = L (one degree, an empty odd class), radii that leave part of a 3- and 4-radius tile,
+# more than 128 north latitudes (two row tiles).
+@pytest.mark.parametrize("L,Ms,Nr", [(31, 31, 8), (32, 16, 9), (33, 11, 7), (47, 24, 6), (191, 95, 8)])
+def test_sliced_transforms(torch, L, Ms, Nr):
+    from paper_2508_16635_gb300 import RotatingShell
+    s = Shell(L, Ms, Nr, 1e-3, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0)
+    x = s.conductive_state() + si.perturbation(L, Ms, Nr, seed=33, amp=3e-2, l_decay=30.0)
+    got = gpu.explicit_terms(torch.tensor(x, device="cuda")).cpu().numpy()
+    want = s.to_real(s.explicit_terms(s.to_complex(x)))
+    assert max(_errors(s, got, want)) < 1e-12
+    # columns of zeros (one field only) and of very different sizes
+    y = x.reshape(3, s.P, Nr, 2).copy()
+    y[0] = 0.0
+    y[1] *= 1e-150
+    got = gpu.explicit_terms(torch.tensor(y.reshape(-1), device="cuda")).cpu().numpy()
+    want = s.to_real(s.explicit_terms(s.to_complex(y.reshape(-1))))
+    assert max(_errors(s, got, want)[1:]) < 1e-12
+    gpu.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_sliced_transforms_pass_on_what_is_not_finite(torch, bad):
+    from paper_2508_16635_gb300 import RotatingShell
+    L, Ms, Nr = 15, 4, 10
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0)
+    U = gpu.conductive_state()
+    U[gpu.phase_slot(Ms, 2) - 1] = bad          # Re T at l = m = M_s
+    U[gpu.n // 3 + 2 * Nr] = 1e-2               # some velocity
+    N = gpu.explicit_terms(U).view(3, gpu.P, Nr, 2)
+    assert not torch.isfinite(N[2, L + 1]).any()
+    gpu.close()
