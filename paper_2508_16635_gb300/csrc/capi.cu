@@ -29,6 +29,7 @@
 #include "chain_cr.cuh"
 #include "products_sym.cuh"
 #include "radial_rhs_f32.cuh"
+#include "radial_rhs_par.cuh"
 #include "cr_factor_gpu.cuh"
 #include "factor_gpu.cuh"
 #include "rsc_internal.h"
@@ -104,6 +105,7 @@ struct rsc_ctx {
   float *f_EdT0 = nullptr, *f_EdT1 = nullptr, *f_EdT2 = nullptr, *f_R0T = nullptr, *f_R1T = nullptr;
   float* f_rd = nullptr;
   float *f_EcT0 = nullptr, *f_EcT2 = nullptr;
+  double *par64[6] = {nullptr}; float* par32[4] = {nullptr};   // ParTables: P0 M0 P1 M1 (irc ird)
   LegDev<double> leg64;
   LegDev<float> leg32;
   // workspace (sized for FP64; the FP32 path uses the front part)
@@ -477,6 +479,44 @@ rsc_status build_ta_tables(rsc_ctx* ctx) {
   return RSC_OK;
 }
 
+// Tables of the radial stages by reflection (radial_rhs_par.cuh): P, M of R0 and R1, 1 / r.
+rsc_status build_par_tables(rsc_ctx* ctx) {
+  const Dims& d = ctx->d;
+  const HostTables& t = ctx->t;
+  const int NH = (d.Nr + 1) / 2, DH = (d.Nd + 1) / 2;
+  for (int o = 0; o < 2; ++o) {
+    const std::vector<double>& Rt = o ? t.R1 : t.R0;
+    std::vector<double> p((size_t)DH * NH), m((size_t)DH * NH);
+    for (int i = 0; i < DH; ++i)
+      for (int j = 0; j < NH; ++j) {
+        const int im = d.Nd - 1 - i;
+        const double a = Rt[(size_t)j * d.Nd + i], b = Rt[(size_t)j * d.Nd + im];
+        // the middle radius of an odd N_d stands alone (folded input a_i, whole entry)
+        p[(size_t)i * NH + j] = im == i ? a : 0.5 * (a + b);
+        m[(size_t)i * NH + j] = im == i ? 0.0 : 0.5 * (a - b);
+      }
+    const std::vector<float> pf(p.begin(), p.end()), mf(m.begin(), m.end());
+    CKS(upload(ctx, &ctx->par64[2 * o], p.data(), p.size()));
+    CKS(upload(ctx, &ctx->par64[2 * o + 1], m.data(), m.size()));
+    CKS(upload(ctx, &ctx->par32[2 * o], pf.data(), pf.size()));
+    CKS(upload(ctx, &ctx->par32[2 * o + 1], mf.data(), mf.size()));
+  }
+  std::vector<double> irc(d.Nr), ird(d.Nd);
+  for (int j = 0; j < d.Nr; ++j) irc[j] = 1.0 / t.rc[j];
+  for (int i = 0; i < d.Nd; ++i) ird[i] = 1.0 / t.rd[i];
+  CKS(upload(ctx, &ctx->par64[4], irc.data(), irc.size()));
+  CKS(upload(ctx, &ctx->par64[5], ird.data(), ird.size()));
+  const int lim = 200 * 1024;
+  for (const void* fn : {(const void*)k_radial_par, (const void*)k_rhs_par<double>, (const void*)k_rhs_par<float>})
+    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  return RSC_OK;
+}
+
+ParTables par_tables(const rsc_ctx* ctx) {
+  return ParTables{ctx->par64[0], ctx->par64[1], ctx->par64[2], ctx->par64[3], ctx->par32[0], ctx->par32[1],
+                   ctx->par32[2], ctx->par32[3], ctx->par64[4], ctx->par64[5], ctx->p.Ra / ctx->d.r_out};
+}
+
 // Digit tables of the FP64 Legendre transforms (slices_tc.cuh), cut on the device from the FP64
 // tables, which nothing else reads and which are released.
 template <bool ANAL>
@@ -549,7 +589,6 @@ rsc_status set_smem_limits(rsc_ctx* ctx) {
   CKS((products_attributes<double, 1>(ctx, big)));
   CKS((products_attributes<float, 1>(ctx, big)));
   CKS((products_attributes<float, 2>(ctx, big)));
-  CK(cudaFuncSetAttribute(k_radial<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   CK(cudaFuncSetAttribute(k_radial<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   {
     // the persistent FP32 radial kernels: one or two blocks per SM with the tables staged
@@ -1058,6 +1097,10 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
       case 2: k_radial_f32<96, 144><<<gr, bl, sm, ctx->s>>>(g, xx, sr); break;
       default: k_radial_f32<0, 0><<<gr, bl, sm, ctx->s>>>(g, xx, sr); break;
     }
+  } else if constexpr (sizeof(R) == 8) {
+    const int ppb = par_pairs((d.Nd + 1) / 2), tw = par_task_threads((d.Nd + 1) / 2);
+    k_radial_par<<<(d.P + ppb - 1) / ppb, 2 * tw, radial_par_smem(d.Nr, d.Nd), ctx->s>>>(
+        g, par_tables(ctx), reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(ctx->SR), ppb);
   } else {
     k_radial<R><<<d.P, round32(std::max(d.Nd, 32)), 3 * d.Nr * sizeof(V), ctx->s>>>(
         g, reinterpret_cast<const double2*>(x), reinterpret_cast<V*>(ctx->SR));
@@ -1217,6 +1260,17 @@ rsc_status stage_rhs(rsc_ctx* ctx, const RhsParams& rp, const double* x, const d
       CK(cudaGetLastError());
       return RSC_OK;
     }
+  }
+  if ((sizeof(R) == 8 || rp.mode != 1) && (!rp.explicit_coriolis || rp.mode == 2)) {
+    // FP64 sums by reflection (k_rhs keeps the explicit Coriolis rows and FP32 Jacobian actions)
+    const double* second = rp.mode == 3 ? (xe && xe != x ? xe : nullptr) : rp.J >= 0 ? U : nullptr;
+    const int ppb = par_pairs((d.Nr + 1) / 2), tw = par_task_threads((d.Nr + 1) / 2);
+    k_rhs_par<R><<<(d.P + ppb - 1) / ppb, (second ? 6 : 4) * tw,
+                   rhs_par_smem(d.Nr, d.Nd, second != nullptr, sizeof(R)), ctx->s>>>(
+        ctx->geom(), rp, par_tables(ctx), reinterpret_cast<const V*>(ctx->AR),
+        reinterpret_cast<const double2*>(x), reinterpret_cast<const double2*>(second), u_orig, out, ppb, tw);
+    CK(cudaGetLastError());
+    return RSC_OK;
   }
   k_rhs<R><<<(d.P + PPB - 1) / PPB, dim3(round32(d.Nr), PPB), smem, ctx->s>>>(
       ctx->geom(), rp, reinterpret_cast<const V*>(ctx->AR), reinterpret_cast<const double2*>(x),
@@ -2370,20 +2424,12 @@ rsc_status tune_precision(rsc_ctx* ctx, rsc_tuning& t, cudaEvent_t e0, cudaEvent
     ctx->tune_ms[1] = timeit([&] { return stage_synth<double>(ctx, ctx->rtmp, ctx->FC); });
     CKS(st);
   }
-  // right-hand side: pairs per block (Jacobian-action mode)
-  RhsParams rp = make_rp(ctx, 200.0, 0.0, 1);
-  best = 1e30;
-  int bp = t.rhs_pairs[p];
-  for (int q : {1, 2, 4, 8}) {
-    if (!threads_fit((const void*)k_rhs<R>, round32(d.Nr) * q) || rhs_smem<R>(d, q) > 200 * 1024)
-      continue;
-    ctx->ppb[p] = q;
-    const double ms = timeit([&] { return stage_rhs<R>(ctx, rp, ctx->rtmp, ctx->rtmp, nullptr, ctx->rhs); });
+  // right-hand side of Jacobian actions (one shape)
+  if (p == 1) {
+    const RhsParams rp = make_rp(ctx, 200.0, 0.0, 1);
+    ctx->tune_ms[2] = timeit([&] { return stage_rhs<R>(ctx, rp, ctx->rtmp, ctx->rtmp, nullptr, ctx->rhs); });
     CKS(st);
-    if (ms < best) { best = ms; bp = q; }
   }
-  ctx->ppb[p] = t.rhs_pairs[p] = bp;
-  if (p == 1) ctx->tune_ms[2] = best;
   return RSC_OK;
 }
 
@@ -2614,6 +2660,7 @@ rsc_status rsc_create(const rsc_params* params, void* stream, rsc_ctx** out) {
   if ((st = set_smem_limits(ctx)) != RSC_OK) return fail(st);
   if ((st = build_tc_tables(ctx)) != RSC_OK) return fail(st);
   if ((st = build_ta_tables(ctx)) != RSC_OK) return fail(st);
+  if ((st = build_par_tables(ctx)) != RSC_OK) return fail(st);
   if ((st = build_slice_tables<false>(ctx)) != RSC_OK) return fail(st);
   if ((st = build_slice_tables<true>(ctx)) != RSC_OK) return fail(st);
   if (cudaMalloc((void**)&ctx->d_status, sizeof(int)) != cudaSuccess ||
@@ -2689,7 +2736,8 @@ rsc_status rsc_destroy(rsc_ctx* ctx) {
                   ctx->f_EdT2, ctx->f_R0T, ctx->f_R1T, ctx->f_rd, ctx->f_EcT0, ctx->f_EcT2, ctx->SR, ctx->FC, ctx->FCU, ctx->UG, ctx->FA,
                   ctx->AR, ctx->rhs, ctx->mid, ctx->xtmp, ctx->vtmp, ctx->rtmp, ctx->ustate, ctx->ref_tmp, ctx->d_Ef[0], ctx->d_Ef[1], ctx->d_Ef[2], ctx->d_Ef[3], ctx->V, ctx->Vs, ctx->partial,
                   ctx->dots, ctx->AR0, ctx->ta_tiles, ctx->ta_off, ctx->cont_hist, ctx->cont_cond, ctx->amax_v, ctx->amax_i, ctx->d_keT, ctx->d_kedT, ctx->d_ker, ctx->d_kew, ctx->d_diag, ctx->d_cr_pairs, ctx->d_E01, ctx->cr_w, ctx->d_cr_rowf, ctx->d_cr_pairf,
-                  ctx->sl[0].tiles, ctx->sl[0].off, ctx->sl[0].ea, ctx->sl[1].tiles, ctx->sl[1].off, ctx->sl[1].ea};
+                  ctx->par64[0], ctx->par64[1], ctx->par64[2], ctx->par64[3], ctx->par64[4], ctx->par64[5],
+                  ctx->par32[0], ctx->par32[1], ctx->par32[2], ctx->par32[3], ctx->sl[0].tiles, ctx->sl[0].off, ctx->sl[0].ea, ctx->sl[1].tiles, ctx->sl[1].off, ctx->sl[1].ea};
   for (void* b : bufs) cudaFree(b);
   for (int q = 0; q < 8; ++q) {
     cudaFree(ctx->leg64.buf[q]);

@@ -81,3 +81,26 @@ def test_sliced_transforms_pass_on_what_is_not_finite(torch, bad):
     N = gpu.explicit_terms(U).view(3, gpu.P, Nr, 2)
     assert not torch.isfinite(N[2, L + 1]).any()
     gpu.close()
+
+
+# Radial stages by reflection: odd and even N_r and N_d (N_r = 6 the smallest, 128 the largest), one
+# and several pairs per block, the last block part full.  The bounds of the explicit terms and of a
+# step and Jacobian action; the second-order step (its boundary rows) 2e-11 as in test_step2_parity.
+@pytest.mark.parametrize("L,Ms,Nr", [(5, 2, 6), (6, 3, 7), (9, 4, 13), (7, 3, 33), (6, 2, 66), (3, 1, 97), (2, 1, 128)])
+def test_radial_stages_by_reflection(torch, L, Ms, Nr):
+    from paper_2508_16635_gb300 import RotatingShell
+    s = Shell(L, Ms, Nr, 1e-3, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0)
+    x = s.conductive_state() + si.perturbation(L, Ms, Nr, seed=35, amp=3e-2)
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    got = gpu.explicit_terms(dev(x)).cpu().numpy()
+    assert max(_errors(s, got, s.to_real(s.explicit_terms(s.to_complex(x))))) < 1e-12
+    got = gpu.step(dev(x), 0.4, 1e-3).cpu().numpy()
+    assert max(_errors(s, got, s.step(x, 0.4, 1e-3))) < 1e-11
+    got = gpu.step2(dev(x), 1e-3).cpu().numpy()
+    assert max(_errors(s, got, s.step2(x, 1e-3))) < 2e-11
+    u = si.random_vector(L, Ms, Nr, seed=36)
+    J = s.real_index("T", Ms, Ms, 1, 1)
+    got = gpu.apply_jacobian(dev(x), 0.4, J, dev(u), 1e-3).cpu().numpy()
+    assert max(_errors(s, got, s.jvp(x, 0.4, J, u, 1e-3))) < 1e-11
+    gpu.close()
