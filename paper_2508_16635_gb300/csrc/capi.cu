@@ -148,10 +148,11 @@ struct rsc_ctx {
                           // per row group (chain_df.cuh), 0 = the FP64 kernels
   int cluster_df = 8;     // CTAs per cluster of the double-float sweeps
   int chain_parts = 1;    // parts per chain of the double-float solve (1: unpartitioned)
+  int nsm = 1;            // SMs of the device
   int chain_cr = 0;       // 1: the double-float solve on odd-even reduced chains (chain_cr.cuh)
   int* d_cr_pairs = nullptr;   // pairs with odd l - m (n_cr_odd), then even (n_cr_even)
   int n_cr_odd = 0, n_cr_even = 0;
-  float4* d_E01 = nullptr;     // [j][k] {E0 hi, E0 lo, E1 hi, E1 lo} at the collocation radii
+  float2* d_E01 = nullptr;     // E0, then E1, [j][k] {hi, lo} at the collocation radii
   float4* d_cr_rowf = nullptr;    // [j] {2 / r^3 hi, lo, 2 / r^2 hi, lo}
   float4* d_cr_pairf = nullptr;   // [p][2] {a l, a}, {c (l + 1), c} (coupling coefficients)
   float4* cr_w = nullptr;      // E0 u, E1 u of the odd blocks, [2][2 P Nr]
@@ -595,6 +596,7 @@ rsc_status set_smem_limits(rsc_ctx* ctx) {
     int dev = 0, nsm = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    ctx->nsm = nsm;
     const Dims& d = ctx->d;
     const size_t lim = 227 * 1024;
     // The attribute belongs to the kernel on this device, not to this context: it only ever
@@ -963,11 +965,12 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
     }
     ctx->n_cr_even = (int)pairs.size() - ctx->n_cr_odd;
     CKS(upload(ctx, &ctx->d_cr_pairs, pairs.data(), pairs.size()));
-    std::vector<float4> e((size_t)d.Nr * d.Nr);
+    std::vector<float2> e(2 * (size_t)d.Nr * d.Nr);
     for (size_t i = 0; i < e.size(); ++i) {
-      const double a = ctx->t.Ec[0][i], b = ctx->t.Ec[1][i];
-      const float ah = (float)a, bh = (float)b;
-      e[i] = make_float4(ah, (float)(a - (double)ah), bh, (float)(b - (double)bh));
+      const size_t nn = (size_t)d.Nr * d.Nr;
+      const double a = i < nn ? ctx->t.Ec[0][i] : ctx->t.Ec[1][i - nn];
+      const float ah = (float)a;
+      e[i] = make_float2(ah, (float)(a - (double)ah));
     }
     CKS(upload(ctx, &ctx->d_E01, e.data(), e.size()));
     auto pair_of = [](double a, double b) {
@@ -1429,34 +1432,36 @@ cudaError_t launch_chain_df(rsc_ctx* ctx, const DevFactor* f, double* out, bool 
 // The passes of the odd-even reduced solve that run over every block (chain_cr.cuh):
 // pass 0 = u and E0 u, E1 u of the odd blocks, 1 = b' and G' b' of the even blocks,
 // 2 = the odd blocks from their neighbours.
-template <int Q>
-void launch_cr_pass_q(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
+template <int CTAS>
+void launch_cr_pass_df(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
   const Dims& d = ctx->d;
   const size_t v = (size_t)d.Nr * sizeof(float4);
   const int* odd = ctx->d_cr_pairs;
   const int* even = ctx->d_cr_pairs + ctx->n_cr_odd;
   double2* o = reinterpret_cast<double2*>(out);
+  // four lanes per row, the rows in equal passes of at most 64
+  const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));
   if (pass == 0)
-    k_cr_odd_df<Q><<<2 * ctx->n_cr_odd, 256, 2 * v, ctx->s>>>(
+    k_cr_odd_df<CTAS><<<2 * ctx->n_cr_odd, thr, 2 * v, ctx->s>>>(
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->rhs, ctx->cr_w);
   else if (pass == 1)
-    k_cr_even_df<Q><<<2 * ctx->n_cr_even, 256, 2 * v, ctx->s>>>(
+    k_cr_even_df<CTAS><<<2 * ctx->n_cr_even, thr, 2 * v, ctx->s>>>(
         ctx->geom(), even, f->cr_red_off, f->Gr, ctx->d_cr_rowf, ctx->d_cr_pairf, ctx->rhs,
         ctx->cr_w, o);
   else
-    k_cr_back_df<Q><<<2 * ctx->n_cr_odd, 256, 5 * v, ctx->s>>>(
+    k_cr_back_df<CTAS><<<2 * ctx->n_cr_odd, thr, 5 * v, ctx->s>>>(
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->d_cr_rowf, ctx->d_cr_pairf,
         ctx->rhs, o);
 }
 
 void launch_cr_pass(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
-  switch (chain_maxq(ctx->d.Nr)) {
-    case 2: launch_cr_pass_q<2>(ctx, f, out, pass); break;
-    case 4: launch_cr_pass_q<4>(ctx, f, out, pass); break;
-    case 8: launch_cr_pass_q<8>(ctx, f, out, pass); break;
-    case 12: launch_cr_pass_q<12>(ctx, f, out, pass); break;
-    default: launch_cr_pass_q<16>(ctx, f, out, pass); break;
-  }
+  const int n = 2 * (pass == 1 ? ctx->n_cr_even : ctx->n_cr_odd);
+  if (n == 0) return;
+  // five CTAs per SM where all are resident at once that way only (chain_cr.cuh)
+  if (n > 4 * ctx->nsm && n <= 5 * ctx->nsm)
+    launch_cr_pass_df<5>(ctx, f, out, pass);
+  else
+    launch_cr_pass_df<4>(ctx, f, out, pass);
 }
 
 void launch_gemv_df(rsc_ctx* ctx, const DevFactor* f, double* out) {

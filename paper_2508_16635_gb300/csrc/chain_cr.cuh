@@ -19,7 +19,17 @@
 // Arithmetic as chain_df.cuh: factor blocks and the tables as double-float pairs
 // {hi, lo} (float4 per complex entry), row sums as Dot2 sums in FP32, vectors FP64 in
 // global memory.  Grid of each kernel: 2 CTAs (e and f block) per pair (m, l) of the given
-// parity of l - m, 256 threads, 8 lanes per row (as k_block_gemv_df).
+// parity of l - m, 4 lanes per row, the rows in equal passes of at most 64.
+//
+// What bounds it: at N_r = 64 every CTA of L = 127, M_s = 12 (748) is resident at once, so the
+// factor blocks' way from HBM (49 MB, 7.4 us) and the sums (48 FP32 instructions per complex entry)
+// overlap little; at N_r = 96, L = 255, M_s = 8 the sums and the 623 MB (93 us) nearly balance.
+// Measured (one GB300, mean of the three passes, us; eight lanes per row, every row of the tables,
+// predicated columns -> this): 27.7 -> 22.4 at L = 127, 185 -> 163 at L = 255, 13.7 -> 11.1 at
+// L = 52, N_r = 60; 32 % fewer instructions.
+// CTAS, the CTAs per SM that the registers allow, is 4 (64 registers: 163 us at L = 255, where 5
+// with 48 registers took 191), and 5 where that puts all of a launch on the device at once and 4
+// does not (22.4 us at L = 127 against 25.3).
 #pragma once
 
 #include "chain_df.cuh"
@@ -80,67 +90,111 @@ __device__ __forceinline__ void cr_axpy(dfl& re, dfl& im, dfl k, float4 v) {
   dfl_fma(im, k.s, k.c, v.y, v.w);
 }
 
+// Start of a kernel: its factor block on the way to L2 while the vectors are prepared.
+__device__ __forceinline__ void cr_prefetch(const float4* M, int Nr) {
+  const char* c = reinterpret_cast<const char*>(M);
+  for (int q = threadIdx.x * 128; q < Nr * Nr * 16; q += blockDim.x * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(c + q));
+}
+
+// Rows are taken in passes of blockDim.x / 4, four lanes per row: a lane's columns are s + 4 q.
+// (Eight lanes per row need a third step of reduction, 14 instructions, for half as many products.)
+constexpr int kCrLanes = 4;
+
+// fn(a, k) per column of a lane: the full groups in chunks of QC, loads first, the rest one by one.
+template <class T, class F>
+__device__ __forceinline__ void cr_columns(const T* __restrict__ row, int s, int Nr, F fn) {
+  constexpr int QC = 4, STEP = QC * kCrLanes;
+  const T* p = row + s;
+  int k = s;
+#pragma unroll 1
+  for (; k - s + STEP <= Nr; k += STEP, p += STEP) {
+    T a[QC];
+#pragma unroll
+    for (int q = 0; q < QC; ++q) a[q] = p[kCrLanes * q];
+#pragma unroll
+    for (int q = 0; q < QC; ++q) fn(a[q], k + kCrLanes * q);
+  }
+#pragma unroll 1
+  for (; k < Nr; k += kCrLanes, p += kCrLanes) fn(*p, k);
+}
+
+// x, y of the lanes of a row: the lane with bit o clear gets x + x of lane ^ o, the other y + y.
+__device__ __forceinline__ dfl cr_pair_sum(dfl x, dfl y, int o) {
+  const bool up = threadIdx.x & o;
+  const dfl keep = up ? y : x, give = up ? x : y;
+  return dfl_add(keep, dfl_shfl_xor(give, o));
+}
+
 // y = M v for one Nr x Nr double-float block M (row-major), v in shared memory; row r of y
-// goes to y[r] (shared memory, packed).  All 256 threads take part; the caller syncs.
-template <int Q>
+// goes to y[r] (shared memory, packed).  All threads take part; the caller syncs.
 __device__ __forceinline__ void cr_gemv(const float4* __restrict__ M, const float4* v, int Nr,
                                         bool real_op, float4* y) {
-  const int s8 = threadIdx.x & 7;
-  const int rows_per_pass = blockDim.x >> 3;
-  for (int r = threadIdx.x >> 3; r < Nr + ((rows_per_pass - Nr % rows_per_pass) % rows_per_pass);
-       r += rows_per_pass) {
-    float4 a[Q];
-    cd_load<Q>(M, r, s8, 0, Nr, r < Nr, a);
-    dfl re0 = dfl_zero(), im0 = dfl_zero(), re1 = dfl_zero(), im1 = dfl_zero();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int k = s8 + 8 * q;
-      if (k < Nr) {
-        if (q & 1)
-          cd_cmac(re1, im1, a[q], v[k], real_op);
-        else
-          cd_cmac(re0, im0, a[q], v[k], real_op);
-      }
+  const int s = threadIdx.x & 3, rows = blockDim.x >> 2;
+  for (int r0 = 0; r0 < Nr; r0 += rows) {
+    const int r = r0 + (threadIdx.x >> 2);
+    if (r0 + ((threadIdx.x & ~31) >> 2) >= Nr) break;   // no row for this warp
+    const float4* row = M + (long)min(r, Nr - 1) * Nr;
+    dfl re = dfl_zero(), im = dfl_zero();
+    if (real_op) {
+      cr_columns(row, s, Nr, [&](float4 a, int k) { cd_cmac(re, im, a, v[k], true); });
+    } else {
+      dfl re1 = dfl_zero(), im1 = dfl_zero();
+      cr_columns(row, s, Nr, [&](float4 a, int k) {
+        const float4 b = v[k];
+        dfl_fma(re, a.x, a.z, b.x, b.z);
+        dfl_fma(im, a.x, a.z, b.y, b.w);
+        dfl_fma(re1, -a.y, -a.w, b.y, b.w);
+        dfl_fma(im1, a.y, a.w, b.x, b.z);
+      });
+      re = dfl_add(re, re1);
+      im = dfl_add(im, im1);
     }
-    dfl re = dfl_add(re0, re1), im = dfl_add(im0, im1);
-    cd_reduce8(re, im);
-    if (r < Nr && s8 == 0) y[r] = cd_pack(re, im);
+    __syncwarp();
+    dfl t = cr_pair_sum(re, im, 1);   // even lanes re, odd lanes im
+    t = dfl_norm(dfl_add(t, dfl_shfl_xor(t, 2)));
+    if (r < Nr && s < 2) {
+      float* o = reinterpret_cast<float*>(y + r) + s;
+      o[0] = t.s;
+      o[2] = t.c;
+    }
   }
 }
 
-// (E0 v0)_j and (E1 v1)_j for every row j (E01[j][k] = {E0 hi, E0 lo, E1 hi, E1 lo}, real),
-// v0, v1 complex double-float in shared memory, packed into e0[j], e1[j] (shared or global).
-template <int Q>
-__device__ __forceinline__ void cr_e01(const float4* __restrict__ E01, const float4* v0,
+// (E0 v0)_j and (E1 v1)_j for every row j (E01: E0, then E1, [j][k] = {hi, lo}, real), v0, v1
+// complex double-float in shared memory, packed into e0[j], e1[j] (shared or global).
+// The radii are symmetric, so T_k and T_k' at row Nr - 1 - j are those at row j times (-1)^k
+// and -(-1)^k: one sum over the even and one over the odd columns give both rows.  A lane's
+// columns s + 4 q have one parity, so the last step of the lanes' reduction joins the two
+// sums, the even lane for row j and the odd one for row Nr - 1 - j.  Tasks: NH rows of E0,
+// NH rows of E1 (whole warps each).
+__device__ __forceinline__ void cr_e01(const float2* __restrict__ E01, const float4* v0,
                                        const float4* v1, int Nr, float4* e0, float4* e1) {
-  const int s8 = threadIdx.x & 7;
-  const int rows_per_pass = blockDim.x >> 3;
-  for (int j = threadIdx.x >> 3; j < Nr + ((rows_per_pass - Nr % rows_per_pass) % rows_per_pass);
-       j += rows_per_pass) {
-    float4 e[Q];
-    cd_load<Q>(E01, j, s8, 0, Nr, j < Nr, e);
-    dfl a = dfl_zero(), b = dfl_zero(), c = dfl_zero(), d = dfl_zero();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int k = s8 + 8 * q;
-      if (k < Nr) {
-        const float4 x = v0[k], y = v1[k];
-        dfl_fma(a, e[q].x, e[q].y, x.x, x.z);
-        dfl_fma(b, e[q].x, e[q].y, x.y, x.w);
-        dfl_fma(c, e[q].z, e[q].w, y.x, y.z);
-        dfl_fma(d, e[q].z, e[q].w, y.y, y.w);
-      }
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-      a = dfl_add(a, dfl_shfl_xor(a, o));
-      b = dfl_add(b, dfl_shfl_xor(b, o));
-      c = dfl_add(c, dfl_shfl_xor(c, o));
-      d = dfl_add(d, dfl_shfl_xor(d, o));
-    }
-    if (j < Nr && s8 == 0) {
-      e0[j] = cd_pack(a, b);
-      e1[j] = cd_pack(c, d);
+  const int s = threadIdx.x & 3, rows = blockDim.x >> 2, NH = (Nr + 1) >> 1, NW = (NH + 7) & ~7;
+  for (int r0 = 0; r0 < 2 * NW; r0 += rows) {
+    const int task = r0 + (threadIdx.x >> 2);
+    if (r0 + ((threadIdx.x & ~31) >> 2) >= 2 * NW) break;
+    const bool one = task >= NW;   // E1
+    const int j = task - (one ? NW : 0);
+    const float2* row = E01 + ((one ? (long)Nr : 0) + min(j, NH - 1)) * Nr;
+    const float4* v = one ? v1 : v0;
+    dfl re = dfl_zero(), im = dfl_zero();
+    cr_columns(row, s, Nr, [&](float2 e, int k) {
+      const float4 x = v[k];
+      dfl_fma(re, e.x, e.y, x.x, x.z);
+      dfl_fma(im, e.x, e.y, x.y, x.w);
+    });
+    __syncwarp();
+    // lanes 0, 1: re of the even and odd columns, lanes 2, 3: im
+    const dfl t = cr_pair_sum(re, im, 2), u = dfl_shfl_xor(t, 1);
+    // row j: even + odd; row Nr - 1 - j: even - odd of E0, odd - even of E1
+    const bool odd = s & 1;
+    const dfl w = dfl_norm(dfl_add(odd && !one ? dfl_neg(t) : t, odd && one ? dfl_neg(u) : u));
+    const int row_out = odd ? Nr - 1 - j : j;
+    if (j < NH && !(odd && row_out == j)) {
+      float* o = reinterpret_cast<float*>((one ? e1 : e0) + row_out) + (s >> 1);
+      o[0] = w.s;
+      o[2] = w.c;
     }
   }
 }
@@ -155,30 +209,31 @@ __device__ __forceinline__ void cr_store(const float4* y, double2* __restrict__ 
 // Odd blocks, first pass: u = D^-1 b, then w0 = E0 u and w1 = E1 u at the block's own rows
 // (w: [2][2 P Nr] float4), for the even neighbours' right-hand sides.
 // Dynamic shared memory: 2 Nr float4.
-template <int Q>
-__global__ void __launch_bounds__(256) k_cr_odd_df(DevGeom g, const int* __restrict__ odd_pairs,
+template <int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_cr_odd_df(DevGeom g, const int* __restrict__ odd_pairs,
                                                    const long* __restrict__ odd_off,
                                                    const float4* __restrict__ Dinv,
-                                                   const float4* __restrict__ E01,
+                                                   const float2* __restrict__ E01,
                                                    const double2* __restrict__ rhs,
                                                    float4* __restrict__ w) {
   extern __shared__ float4 cr_sh[];
   const int Nr = g.Nr;
   const CrBlock b = cr_block(g, odd_pairs);
+  const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
+  cr_prefetch(Di, Nr);
   float4* sb = cr_sh;
   float4* su = cr_sh + Nr;
   for (int k = threadIdx.x; k < Nr; k += blockDim.x) sb[k] = cd_split(rhs[b.row0 + k]);
   __syncthreads();
-  const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
-  cr_gemv<Q>(Di, sb, Nr, b.m == 0, su);
+  cr_gemv(Di, sb, Nr, b.m == 0, su);
   __syncthreads();
-  cr_e01<Q>(E01, su, su, Nr, w + b.row0, w + 2L * g.P * Nr + b.row0);
+  cr_e01(E01, su, su, Nr, w + b.row0, w + 2L * g.P * Nr + b.row0);
 }
 
 // Even blocks: b' = b - A u_{i-1} - C u_{i+1} from the neighbours' w, then g' = G' b' into
 // out.  Dynamic shared memory: 2 Nr float4.
-template <int Q>
-__global__ void __launch_bounds__(256) k_cr_even_df(DevGeom g, const int* __restrict__ even_pairs,
+template <int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_cr_even_df(DevGeom g, const int* __restrict__ even_pairs,
                                                     const long* __restrict__ red_off,
                                                     const float4* __restrict__ Gr,
                                                     const float4* __restrict__ rowf,
@@ -189,6 +244,8 @@ __global__ void __launch_bounds__(256) k_cr_even_df(DevGeom g, const int* __rest
   extern __shared__ float4 cr_sh[];
   const int Nr = g.Nr;
   const CrBlock b = cr_block(g, even_pairs);
+  const float4* Gt = Gr + (red_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
+  cr_prefetch(Gt, Nr);
   float4* sb = cr_sh;
   float4* sy = cr_sh + Nr;
   const long half = 2L * g.P * Nr;
@@ -215,8 +272,7 @@ __global__ void __launch_bounds__(256) k_cr_even_df(DevGeom g, const int* __rest
     sb[j] = cd_pack(re, im);
   }
   __syncthreads();
-  const float4* Gt = Gr + (red_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
-  cr_gemv<Q>(Gt, sb, Nr, b.m == 0, sy);
+  cr_gemv(Gt, sb, Nr, b.m == 0, sy);
   __syncthreads();
   cr_store(sy, out, b.row0, Nr);
 }
@@ -226,11 +282,11 @@ __global__ void __launch_bounds__(256) k_cr_even_df(DevGeom g, const int* __rest
 //   A x_{i-1} + C x_{i+1} = s ir E0 y0 - s E1 y1,
 //   y0 = a l x_{i-1} - c (l + 1) x_{i+1},   y1 = a x_{i-1} + c x_{i+1}:
 // two table products per block.  Dynamic shared memory: 5 Nr float4.
-template <int Q>
-__global__ void __launch_bounds__(256) k_cr_back_df(DevGeom g, const int* __restrict__ odd_pairs,
+template <int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_cr_back_df(DevGeom g, const int* __restrict__ odd_pairs,
                                                     const long* __restrict__ odd_off,
                                                     const float4* __restrict__ Dinv,
-                                                    const float4* __restrict__ E01,
+                                                    const float2* __restrict__ E01,
                                                     const float4* __restrict__ rowf,
                                                     const float4* __restrict__ pairf,
                                                     const double2* __restrict__ rhs,
@@ -238,6 +294,8 @@ __global__ void __launch_bounds__(256) k_cr_back_df(DevGeom g, const int* __rest
   extern __shared__ float4 cr_sh[];
   const int Nr = g.Nr;
   const CrBlock b = cr_block(g, odd_pairs);
+  const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
+  cr_prefetch(Di, Nr);
   float4* y0 = cr_sh;
   float4* y1 = cr_sh + Nr;
   float4* e0 = cr_sh + 2 * Nr;
@@ -261,7 +319,7 @@ __global__ void __launch_bounds__(256) k_cr_back_df(DevGeom g, const int* __rest
     y1[k] = cd_pack(r1, i1);
   }
   __syncthreads();
-  cr_e01<Q>(E01, y0, y1, Nr, e0, e1);
+  cr_e01(E01, y0, y1, Nr, e0, e1);
   __syncthreads();
   for (int j = threadIdx.x; j < Nr; j += blockDim.x) {
     const double2 bv = rhs[b.row0 + j];
@@ -274,8 +332,7 @@ __global__ void __launch_bounds__(256) k_cr_back_df(DevGeom g, const int* __rest
     sr[j] = cd_pack(re, im);
   }
   __syncthreads();
-  const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
-  cr_gemv<Q>(Di, sr, Nr, b.m == 0, y0);
+  cr_gemv(Di, sr, Nr, b.m == 0, y0);
   __syncthreads();
   cr_store(y0, out, b.row0, Nr);
 }

@@ -85,8 +85,8 @@ RSC_HD void dfl_fma(dfl& a, float xh, float xl, float yh, float yl) {
   const float t = df_add(a.s, p);
   const float z = df_add(t, -a.s);
   const float err = df_add(df_add(a.s, -df_add(t, -z)), df_add(p, -z));
-  const float cross = df_fma(xh, yl, df_mul(xl, yh));
-  a.c = df_add(a.c, df_add(err, df_add(e, cross)));
+  const float cross = df_fma(xh, yl, df_fma(xl, yh, e));
+  a.c = df_add(a.c, df_add(err, cross));
   a.s = t;
 }
 

@@ -104,3 +104,24 @@ def test_radial_stages_by_reflection(torch, L, Ms, Nr):
     got = gpu.apply_jacobian(dev(x), 0.4, J, dev(u), 1e-3).cpu().numpy()
     assert max(_errors(s, got, s.jvp(x, 0.4, J, u, 1e-3))) < 1e-11
     gpu.close()
+
+
+# Passes of the odd-even reduced chain solve: rows that fill part of a warp, one, two passes of
+# rows, columns that end inside a chunk, odd N_r (a middle row of its own), a chain of one and of two
+# blocks (no even or odd neighbour), and 612 CTAs (between four and five per SM of 152).  Bounds as
+# test_implicit_solve_backward_error_* of test_gpu_parity.py.
+@pytest.mark.parametrize("L,Ms,Nr", [(4, 4, 6), (9, 3, 17), (12, 5, 33), (7, 7, 64), (8, 8, 65),
+                                     (5, 4, 128), (34, 1, 8)])
+@pytest.mark.parametrize("precision", ["mixed"])
+def test_reduced_chain_passes(torch, L, Ms, Nr, precision):
+    from paper_2508_16635_gb300 import RotatingShell
+    from tests.test_gpu_parity import U48, _random_rhs, _solve_errors
+    s = Shell(L, Ms, Nr, 1e-3, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0, precision=precision)
+    b = _random_rhs(s, 41)
+    x = gpu.implicit_solve(torch.tensor(s.to_real(b), device="cuda"), 2e-3).cpu().numpy()
+    eta, fwd, fwd_T = _solve_errors(s, 2e-3, b, s.to_complex(x))
+    assert eta < 64 * U48
+    assert fwd < 32 * 1e-10
+    assert fwd_T < 1e-12
+    gpu.close()
