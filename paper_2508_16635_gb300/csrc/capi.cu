@@ -1618,12 +1618,12 @@ rsc_status stage_solve_fp64(rsc_ctx* ctx, const DevFactor* f, double* out) {
   int nb;
   launch_1d_grid(nef, &nb);
   for (int it = 0; it < ctx->refine; ++it) {
-    {
+    {   // the residual r is in place over b: the next one is r less the operator of the last correction
       KSpan sp(ctx, RSC_K_CHAIN, 3.0 * d.n() * 8.0 + 4.0 * d.Nr * d.Nr * 8.0,
                2.0 * d.P * d.Nr * d.Nr * 12.0);
       k_chain_residual<<<d.P, dim3(round32(d.Nr), 2), 6 * (size_t)d.Nr * sizeof(double2), ctx->s>>>(
           fac_geom(ctx, f->dt), ctx->d_pair_l, ctx->d_pair_m, d.P,
-          reinterpret_cast<const double2*>(out), ctx->rhs);
+          reinterpret_cast<const double2*>(it ? ctx->ref_tmp : out), ctx->rhs);
       CK(cudaGetLastError());
     }
     CKS(stage_solve(ctx, f, ctx->ref_tmp, false, false));

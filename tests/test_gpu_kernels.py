@@ -125,3 +125,24 @@ def test_reduced_chain_passes(torch, L, Ms, Nr, precision):
     assert fwd < 32 * 1e-10
     assert fwd_T < 1e-12
     gpu.close()
+
+
+# Residual of the refined FP64 solve: rows in pairs (odd N_r: a middle row alone), row pairs that fill
+# part of a warp, pairs past the last block.  A second refinement leaves the solution where the first
+# puts it (within the bounds of the FP64 solve in test_gpu_parity.py): a wrong residual moves it by O(1).
+@pytest.mark.parametrize("L,Ms,Nr", [(4, 4, 6), (9, 3, 17), (13, 1, 33), (7, 7, 64), (8, 8, 65), (5, 4, 128)])
+def test_chain_residual(torch, L, Ms, Nr):
+    from paper_2508_16635_gb300 import RotatingShell
+    from tests.test_gpu_parity import U64, _random_rhs, _solve_errors
+    s = Shell(L, Ms, Nr, 1e-4, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-4, 80.0)
+    b = _random_rhs(s, 43)
+    B = torch.tensor(s.to_real(b), device="cuda")
+    t0 = gpu.tuning()
+    for refine in (1, 2):
+        gpu.set_tuning(dict(t0, refine=refine))
+        eta, fwd, fwd_T = _solve_errors(s, 2e-3, b, s.to_complex(gpu.implicit_solve(B, 2e-3).cpu().numpy()))
+        assert eta < 64 * U64
+        assert fwd < 1e-11
+        assert fwd_T < 1e-12
+    gpu.close()
