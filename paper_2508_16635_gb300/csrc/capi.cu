@@ -100,7 +100,7 @@ struct rsc_ctx {
   int *d_m_of = nullptr, *d_pstart = nullptr, *d_pair_l = nullptr, *d_pair_m = nullptr;
   long* d_leg_off = nullptr;
   double *d_rc = nullptr, *d_rd = nullptr, *d_EcT0 = nullptr, *d_EcT2 = nullptr;
-  double* d_EcT1 = nullptr;
+  double *d_EcT1 = nullptr, *d_EcT4 = nullptr;
   double *d_EdT0 = nullptr, *d_EdT1 = nullptr, *d_EdT2 = nullptr, *d_R0T = nullptr, *d_R1T = nullptr;
   float *f_EdT0 = nullptr, *f_EdT1 = nullptr, *f_EdT2 = nullptr, *f_R0T = nullptr, *f_R1T = nullptr;
   float* f_rd = nullptr;
@@ -122,6 +122,7 @@ struct rsc_ctx {
   int factor_gpu = 1;          // 1: factorise on the GPU (k_factor_*), 0: on the host
   int refine = 1;              // iterative-refinement steps of every FP64 e/f chain solve
   double* ref_tmp = nullptr;   // correction of a refinement step
+  double2* res_z = nullptr;    // table products of its residual, [7][P][Nr]
   double factor_s = 0.0;       // wall time of the last factorisation (s)
   int factor_on_gpu = 0;       // where the last factorisation ran
   double factor_cr_s = 0.0;    // the same for the last factorisation of the reduced chains
@@ -153,6 +154,8 @@ struct rsc_ctx {
   int* d_cr_pairs = nullptr;   // pairs with odd l - m (n_cr_odd), then even (n_cr_even)
   int n_cr_odd = 0, n_cr_even = 0;
   float2* d_E01 = nullptr;     // E0, then E1, [j][k] {hi, lo} at the collocation radii
+  double2* d_rowf64 = nullptr;    // [j] {2 / r^3, 2 / r^2}
+  CrPair* d_pairf64 = nullptr;    // [p] {a l, a, c (l + 1), c}
   float4* d_cr_rowf = nullptr;    // [j] {2 / r^3 hi, lo, 2 / r^2 hi, lo}
   float4* d_cr_pairf = nullptr;   // [p][2] {a l, a}, {c (l + 1), c} (coupling coefficients)
   float4* cr_w = nullptr;      // E0 u, E1 u of the odd blocks, [2][2 P Nr]
@@ -481,6 +484,14 @@ rsc_status build_ta_tables(rsc_ctx* ctx) {
 }
 
 // Tables of the radial stages by reflection (radial_rhs_par.cuh): P, M of R0 and R1, 1 / r.
+// Normalised coefficients of the couplings to l - 1 and l + 1 (Eqs. impcor_e_final /
+// impcor_f_final, the N_l^m ratio folded in).
+void coupling_factors(double l, double m, double (&k)[2]) {
+  const double l1 = l + 1.0;
+  k[0] = l == 0 ? 0.0 : (l * l - 1.0) * std::sqrt((l * l - m * m) / (4.0 * l * l - 1.0));
+  k[1] = l == 0 ? 0.0 : l * (l + 2.0) * std::sqrt((l1 * l1 - m * m) / (4.0 * l1 * l1 - 1.0));
+}
+
 rsc_status build_par_tables(rsc_ctx* ctx) {
   const Dims& d = ctx->d;
   const HostTables& t = ctx->t;
@@ -507,6 +518,21 @@ rsc_status build_par_tables(rsc_ctx* ctx) {
   for (int i = 0; i < d.Nd; ++i) ird[i] = 1.0 / t.rd[i];
   CKS(upload(ctx, &ctx->par64[4], irc.data(), irc.size()));
   CKS(upload(ctx, &ctx->par64[5], ird.data(), ird.size()));
+  // factors of the Coriolis couplings (CrPair): those of the reduced chains, in FP64
+  std::vector<double2> rowf(d.Nr);
+  std::vector<CrPair> pairf(d.P);
+  for (int j = 0; j < d.Nr; ++j) {
+    const double r = t.rc[j], sc = 2.0 / (r * r);
+    rowf[j] = make_double2(sc / r, sc);
+  }
+  for (int p = 0; p < d.P; ++p) {
+    double k[2];
+    coupling_factors(t.pair_l[p], t.pair_m[p], k);
+    const double l = t.pair_l[p];
+    pairf[p] = {k[0] * l, k[0], k[1] * (l + 1.0), k[1]};
+  }
+  CKS(upload(ctx, &ctx->d_rowf64, rowf.data(), rowf.size()));
+  CKS(upload(ctx, &ctx->d_pairf64, pairf.data(), pairf.size()));
   const int lim = 200 * 1024;
   for (const void* fn : {(const void*)k_radial_par, (const void*)k_rhs_par<double>, (const void*)k_rhs_par<float>})
     CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
@@ -982,14 +1008,12 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
       const double r = ctx->t.rc[j], sc = 2.0 / (r * r);
       rowf[j] = pair_of(sc / r, sc);
     }
-    // normalised coefficients of the couplings to l - 1 and l + 1 (Eqs. impcor_e_final /
-    // impcor_f_final, the N_l^m ratio folded in)
     for (int p = 0; p < d.P; ++p) {
-      const double l = ctx->t.pair_l[p], m = ctx->t.pair_m[p], l1 = l + 1.0;
-      const double a = l == 0 ? 0.0 : (l * l - 1.0) * std::sqrt((l * l - m * m) / (4.0 * l * l - 1.0));
-      const double c = l == 0 ? 0.0 : l * (l + 2.0) * std::sqrt((l1 * l1 - m * m) / (4.0 * l1 * l1 - 1.0));
-      pairf[2 * p] = pair_of(a * l, a);
-      pairf[2 * p + 1] = pair_of(c * l1, c);
+      double k[2];
+      coupling_factors(ctx->t.pair_l[p], ctx->t.pair_m[p], k);
+      const double l = ctx->t.pair_l[p];
+      pairf[2 * p] = pair_of(k[0] * l, k[0]);
+      pairf[2 * p + 1] = pair_of(k[1] * (l + 1.0), k[1]);
     }
     CKS(upload(ctx, &ctx->d_cr_rowf, rowf.data(), rowf.size()));
     CKS(upload(ctx, &ctx->d_cr_pairf, pairf.data(), pairf.size()));
@@ -1618,12 +1642,19 @@ rsc_status stage_solve_fp64(rsc_ctx* ctx, const DevFactor* f, double* out) {
   int nb;
   launch_1d_grid(nef, &nb);
   for (int it = 0; it < ctx->refine; ++it) {
-    {   // the residual r is in place over b: the next one is r less the operator of the last correction
+    {
       KSpan sp(ctx, RSC_K_CHAIN, 3.0 * d.n() * 8.0 + 4.0 * d.Nr * d.Nr * 8.0,
                2.0 * d.P * d.Nr * d.Nr * 12.0);
-      k_chain_residual<<<d.P, dim3(round32(d.Nr), 2), 6 * (size_t)d.Nr * sizeof(double2), ctx->s>>>(
-          fac_geom(ctx, f->dt), ctx->d_pair_l, ctx->d_pair_m, d.P,
-          reinterpret_cast<const double2*>(it ? ctx->ref_tmp : out), ctx->rhs);
+      const int NH = (d.Nr + 1) / 2, ppb = par_pairs(NH), tw = par_task_threads(NH);
+      const FacGeom fg = fac_geom(ctx, f->dt);
+      // the residual r is in place over b: the next one is r less the operator of the last correction
+      const double2* xo = reinterpret_cast<const double2*>(it ? ctx->ref_tmp : out);
+      k_chain_products<<<(d.P + ppb - 1) / ppb, 4 * tw, 4 * (size_t)ppb * d.Nr * sizeof(double), ctx->s>>>(
+          fg, ctx->d_EcT0, ctx->d_EcT1, ctx->d_EcT2, ctx->d_EcT4, d.P, xo, ctx->res_z, ppb);
+      CK(cudaGetLastError());
+      k_chain_residual<<<(int)(((long)d.P * d.Nr + 127) / 128), 128, 0, ctx->s>>>(
+          fg, ctx->par64[4], ctx->d_rowf64, ctx->d_pairf64, ctx->d_pair_l, ctx->d_pair_m, d.P, ctx->res_z, xo,
+          ctx->rhs);
       CK(cudaGetLastError());
     }
     CKS(stage_solve(ctx, f, ctx->ref_tmp, false, false));
@@ -2633,6 +2664,8 @@ rsc_status rsc_create(const rsc_params* params, void* stream, rsc_ctx** out) {
     auto e0 = transpose(t.Ec[0], d.Nr, d.Nr), e2 = transpose(t.Ec[2], d.Nr, d.Nr);
     auto e1 = transpose(t.Ec[1], d.Nr, d.Nr);
     UP(ctx->d_EcT1, e1);
+    auto e4 = transpose(t.Ec[4], d.Nr, d.Nr);
+    UP(ctx->d_EcT4, e4);
     UP(ctx->d_Ef[0], t.Ec[0]);
     UP(ctx->d_Ef[1], t.Ec[1]);
     UP(ctx->d_Ef[2], t.Ec[2]);
@@ -2713,6 +2746,7 @@ rsc_status rsc_create(const rsc_params* params, void* stream, rsc_ctx** out) {
   if ((st = alloc((void**)&ctx->rtmp, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
   if ((st = alloc((void**)&ctx->ustate, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
   if ((st = alloc((void**)&ctx->ref_tmp, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
+  if ((st = alloc((void**)&ctx->res_z, 7 * (size_t)d.P * d.Nr * c16)) != RSC_OK) return fail(st);
   ctx->nblk_dot = (int)std::max<long>((n + 1023) / 1024, 152L * 8);   // pass-A chunks, pass-B blocks
   if ((st = alloc((void**)&ctx->partial, (size_t)ctx->nblk_dot * (2 * kMaxKrylov + 4) * sizeof(double))) != RSC_OK)
     return fail(st);
@@ -2735,7 +2769,7 @@ rsc_status rsc_destroy(rsc_ctx* ctx) {
   if (ctx->s2) cudaStreamSynchronize(ctx->s2), cudaStreamDestroy(ctx->s2);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
+  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_EcT4, ctx->res_z, ctx->d_rowf64, ctx->d_pairf64, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
                   ctx->d_rc, ctx->d_rd, ctx->d_EcT0, ctx->d_EcT2, ctx->d_EdT0, ctx->d_EdT1,
                   ctx->d_EdT2, ctx->d_R0T, ctx->d_R1T, ctx->f_EdT0, ctx->f_EdT1,
                   ctx->f_EdT2, ctx->f_R0T, ctx->f_R1T, ctx->f_rd, ctx->f_EcT0, ctx->f_EcT2, ctx->SR, ctx->FC, ctx->FCU, ctx->UG, ctx->FA,

@@ -459,93 +459,138 @@ __global__ void __launch_bounds__(kFacThreads) k_factor_temp(FacGeom g, double* 
 
 // Residual of the e/f chains, for iterative refinement of the FP64 chain solve:
 // r = b - (M/dt + K) x on the e and f rows (the operator of fac_diag / fac_coupling_row
-// applied to x through the Chebyshev tables: D x needs E0 x, E1 x, E2 x, E4 x of the
-// pair's own coefficients, the couplings E0 x and E1 x of the other potential at l - 1 and
-// l + 1), in place over rb (b on entry, r on exit); the temperature rows are set to 0.
+// applied to x through the Chebyshev tables), in place over rb (b on entry, r on exit); the
+// temperature rows are set to 0.
 // The block Thomas sweeps multiply by explicit block inverses, which is not backward
 // stable: at Ek = 1e-5 the small poloidal field f of the m = 0 chains can carry relative
 // errors of 1e-8.  One refinement step x += solve(r) with this FP64 residual brings the
 // solution to the accuracy of a pivoted banded LU (1e-15 on the same chains).
-// grid = P (one CTA per pair), block = (round32(Nr), 2): threadIdx.y = field e / f.
-__global__ void k_chain_residual(FacGeom g, const int* __restrict__ pair_l,
-                                 const int* __restrict__ pair_m, int P,
-                                 const double2* __restrict__ x, double2* __restrict__ rb) {
-  extern __shared__ double2 xs_[];   // [fld][pair offset -1, 0, +1][Nr]
-  const int Nr = g.Nr, p = blockIdx.x;
-  const int l = pair_l[p], m = pair_m[p];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
-  for (int idx = tid; idx < 6 * Nr; idx += nt) {
-    const int fld = idx / (3 * Nr), o = (idx / Nr) % 3 - 1, k = idx % Nr;
-    const int l2 = l + o;
-    double2 v = make_double2(0.0, 0.0);
-    if (l2 >= m && l2 <= g.L) v = x[((long)fld * P + p + o) * Nr + k];
-    xs_[idx] = v;
+//
+// Two kernels: the table products E0, E1, E2 e and E0, E1, E2, E4 f of every pair once (a pair's
+// couplings to l - 1 and l + 1 need E0 and E1 of its neighbours, which one kernel summed again),
+// two rows j and Nr - 1 - j at a time by the parity of T_k; then the rows from them.  Both FP64;
+// bound by the FP64 pipe (4.1 times fewer multiply-adds than summing per row and coupling).
+// Measured at L = 127, M_s = 12, N_r = 64: 198 -> 64 us per residual on one GB300.
+
+// Coupling factors of pair p (chain_cr.cuh): {a l, a, c (l + 1), c}.
+struct __align__(16) CrPair {
+  double x, y, z, w;
+};
+
+// Z[(q P + p) Nr + j], q = E0 e, E1 e, E2 e, E0 f, E1 f, E2 f, E4 f.
+// grid = ceil(P / PPB), block = 4 TW: thread group = thread / TW: e re, e im, f re, f im; thread l of a
+// group = (pair l / NH, row l % NH) of the block, NH = ceil(Nr / 2).  Shared memory 4 PPB Nr doubles.
+__global__ void __launch_bounds__(640) k_chain_products(FacGeom g, const double* __restrict__ E0T,
+                                                        const double* __restrict__ E1T,
+                                                        const double* __restrict__ E2T,
+                                                        const double* __restrict__ E4T, int P,
+                                                        const double2* __restrict__ x, double2* __restrict__ Z,
+                                                        int PPB) {
+  extern __shared__ double cp_sh[];   // [group][pl][k]
+  const int Nr = g.Nr, NH = (Nr + 1) / 2;
+  const int pb = blockIdx.x * PPB, np = min(PPB, P - pb);
+  for (int idx = threadIdx.x; idx < 2 * np * Nr; idx += blockDim.x) {
+    const int f = idx / (np * Nr), r = idx - f * np * Nr;
+    const double2 v = x[((long)f * P + pb) * Nr + r];
+    cp_sh[2 * f * PPB * Nr + r] = v.x;
+    cp_sh[(2 * f + 1) * PPB * Nr + r] = v.y;
   }
   __syncthreads();
-  const int j = threadIdx.x, fld = threadIdx.y;
-  if (j >= Nr) return;
-  const long row = ((long)fld * P + p) * Nr + j;
-  if (fld == 0) rb[((long)2 * P + p) * Nr + j] = make_double2(0.0, 0.0);
-  const double2* xo = xs_ + (fld * 3 + 1) * Nr;   // own coefficients at l
-  double2 Ax;
+  const int TW = blockDim.x >> 2, grp = threadIdx.x / TW, l = threadIdx.x - grp * TW;
+  const int pl = l / NH, jj = l - pl * NH, f = grp >> 1;
+  if (pl >= np) return;
+  const double* v = cp_sh + (grp * PPB + pl) * Nr;
+  double se[4] = {0, 0, 0, 0}, so[4] = {0, 0, 0, 0};
+  auto step = [&](double (&s)[4], int k) {
+    const double a = v[k];
+    const long o = (long)k * Nr + jj;
+    s[0] = fma(E0T[o], a, s[0]);
+    s[1] = fma(E1T[o], a, s[1]);
+    s[2] = fma(E2T[o], a, s[2]);
+    if (f) s[3] = fma(E4T[o], a, s[3]);
+  };
+  for (int k = 0; k + 1 < Nr; k += 2) {
+    step(se, k);
+    step(so, k + 1);
+  }
+  if (Nr & 1) step(se, Nr - 1);
+  double* z = reinterpret_cast<double*>(Z) + (grp & 1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (q == 3 && !f) break;
+    double* o = z + 2 * (((long)(3 * f + q) * P + pb + pl) * Nr);
+    o[2 * jj] = se[q] + so[q];
+    o[2 * (Nr - 1 - jj)] = q == 1 ? so[q] - se[q] : se[q] - so[q];   // the odd derivative changes sign
+  }
+}
+
+// The rows, one thread per (pair, row j); rowf[j] = {2 / r^3, 2 / r^2}, pairf: CrPair.
+// (Reciprocals and coupling coefficients from tables: an FP64 division or square root is some twenty
+// instructions of the narrow pipe.)
+__global__ void k_chain_residual(FacGeom g, const double* __restrict__ irc, const double2* __restrict__ rowf,
+                                 const CrPair* __restrict__ pairf, const int* __restrict__ pair_l,
+                                 const int* __restrict__ pair_m, int P, const double2* __restrict__ Z,
+                                 const double2* __restrict__ x, double2* __restrict__ rb) {
+  const int Nr = g.Nr;
+  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long)P * Nr) return;
+  const int p = (int)(idx / Nr), j = (int)(idx - (long)p * Nr);
+  const int l = pair_l[p], m = pair_m[p];
+  const long np = (long)P * Nr;
+  rb[2 * np + idx] = make_double2(0.0, 0.0);
+  const double ir = irc[j], ir2 = ir * ir, lam = l * (l + 1.0), mk = lam * g.Ek * ir2;
+  auto sub = [&](int fld, double2 a) {
+    const double2 b = rb[fld * np + idx];
+    rb[fld * np + idx] = make_double2(b.x - a.x, b.y - a.y);
+  };
   if (l == 0) {
-    Ax = xo[j];
-  } else {
-    double2 e0 = {0, 0}, e1 = {0, 0}, e2 = {0, 0}, e4 = {0, 0};
-    // rows of the tables: interior rows use row j; the boundary rows their wall rows
-    const bool bc = (j == 0 || j == Nr - 1) || (fld == 1 && (j == 1 || j == Nr - 2));
-    const int jr = (j <= 1) ? 0 : (j >= Nr - 2 ? Nr - 1 : j);
-    const int rr = bc ? jr : j;
-    for (int k = 0; k < Nr; ++k) {
-      const size_t rk = (size_t)rr * Nr + k;
-      const double2 v = xo[k];
-      const double c0 = g.E0[rk], c1 = g.E1[rk];
-      e0.x = fma(c0, v.x, e0.x); e0.y = fma(c0, v.y, e0.y);
-      e1.x = fma(c1, v.x, e1.x); e1.y = fma(c1, v.y, e1.y);
-      if (!bc) {
-        const double c2 = g.E2[rk], c4 = g.E4[rk];
-        e2.x = fma(c2, v.x, e2.x); e2.y = fma(c2, v.y, e2.y);
-        e4.x = fma(c4, v.x, e4.x); e4.y = fma(c4, v.y, e4.y);
-      }
-    }
-    if (bc) {
-      Ax = (j == 0 || j == Nr - 1) ? e0 : e1;   // f: rows 1, Nr - 2 hold d_r f at the walls
+    sub(0, x[idx]);
+    sub(1, x[np + idx]);
+    return;
+  }
+#pragma unroll
+  for (int fld = 0; fld < 2; ++fld) {
+    const double2* z = Z + (fld ? 3 : 0) * np;
+    double2 Ax;
+    if (j == 0 || j == Nr - 1) {
+      Ax = z[idx];
+    } else if (fld == 1 && (j == 1 || j == Nr - 2)) {
+      Ax = z[np + idx + (j == 1 ? -1 : 1)];   // rows 1, Nr - 2 hold d_r f at the walls
     } else {
-      const double r = g.rc[j], r2 = r * r, lam = l * (l + 1.0), mk = lam * g.Ek / r2;
-      const double2 Ll = make_double2(e2.x - lam / r2 * e0.x, e2.y - lam / r2 * e0.y);
+      const double2 e0 = z[idx], e2 = z[2 * np + idx];
+      const double2 Ll = make_double2(e2.x - lam * ir2 * e0.x, e2.y - lam * ir2 * e0.y);
       if (fld == 0) {
-        const double cm = g.explicit_coriolis ? 0.0 : -2.0 * m / r2;   // times i e
+        const double cm = g.explicit_coriolis ? 0.0 : -2.0 * m * ir2;   // times i e
         Ax = make_double2(mk * g.inv_dt * e0.x - mk * Ll.x - cm * e0.y,
                           mk * g.inv_dt * e0.y - mk * Ll.y + cm * e0.x);
       } else {
-        const double c2 = -2.0 * lam / r2, c1 = 4.0 * lam / (r2 * r), c0 = (lam * lam - 6.0 * lam) / (r2 * r2);
+        const double2 e1 = z[np + idx], e4 = z[3 * np + idx];
+        const double c2 = -2.0 * lam * ir2, c1 = 4.0 * lam * (ir2 * ir), c0 = (lam * lam - 6.0 * lam) * (ir2 * ir2);
         const double2 LL = make_double2(e4.x + c2 * e2.x + c1 * e1.x + c0 * e0.x,
                                         e4.y + c2 * e2.y + c1 * e1.y + c0 * e0.y);
-        const double cm = g.explicit_coriolis ? 0.0 : 2.0 * m / r2;     // times i Ll f
+        const double cm = g.explicit_coriolis ? 0.0 : 2.0 * m * ir2;     // times i Ll f
         Ax = make_double2(-mk * g.inv_dt * Ll.x + mk * LL.x - cm * Ll.y,
                           -mk * g.inv_dt * Ll.y + mk * LL.y + cm * Ll.x);
       }
-      // Coriolis couplings to the other potential at l - 1 and l + 1
-      for (int side = -1; side <= 1; side += 2) {
-        if ((side < 0 && l - 1 < m) || (side > 0 && l + 1 > g.L)) continue;
-        double a2, al;
-        fac_coupling_row(g, fld, l, m, side, j, a2, al);
-        if (a2 == 0.0) continue;
-        const double2* xn = xs_ + ((1 - fld) * 3 + 1 + side) * Nr;
-        double2 n0 = {0, 0}, n1 = {0, 0};
-        for (int k = 0; k < Nr; ++k) {
-          const size_t jk = (size_t)j * Nr + k;
-          const double c0 = g.E0[jk], c1 = g.E1[jk];
-          n0.x = fma(c0, xn[k].x, n0.x); n0.y = fma(c0, xn[k].y, n0.y);
-          n1.x = fma(c1, xn[k].x, n1.x); n1.y = fma(c1, xn[k].y, n1.y);
+      // Coriolis couplings to the other potential at l - 1 and l + 1 (this row carries them)
+      if (!g.explicit_coriolis) {
+        const double2* n = Z + (fld ? 0 : 3) * np + idx;
+        const double2 rf = rowf[j];
+        const CrPair pf = pairf[p];
+        if (l - 1 >= m) {
+          const double2 n0 = n[-Nr], n1 = n[np - Nr];
+          Ax.x += rf.x * (pf.x * n0.x) - rf.y * (pf.y * n1.x);
+          Ax.y += rf.x * (pf.x * n0.y) - rf.y * (pf.y * n1.y);
         }
-        Ax.x += a2 * (al * n0.x - n1.x);
-        Ax.y += a2 * (al * n0.y - n1.y);
+        if (l + 1 <= g.L) {
+          const double2 n0 = n[Nr], n1 = n[np + Nr];
+          Ax.x -= rf.x * (pf.z * n0.x) + rf.y * (pf.w * n1.x);
+          Ax.y -= rf.x * (pf.z * n0.y) + rf.y * (pf.w * n1.y);
+        }
       }
     }
+    sub(fld, Ax);
   }
-  const double2 b = rb[row];
-  rb[row] = make_double2(b.x - Ax.x, b.y - Ax.y);
 }
 
 // Double-float copies of the factors for the mixed path: hi = the entry rounded to FP32,
