@@ -175,8 +175,8 @@ rsc_status rsc_explicit_terms(rsc_ctx* ctx, const double* U, double* N);
  * use.  Returns RSC_EINVAL for a null pointer or dt <= 0.                   */
 rsc_status rsc_implicit_solve(rsc_ctx* ctx, const double* rhs, double* x, double dt);
 
-/* One block of the factorisation of dt (built first if needed), copied to the host
- * (synchronous).  which = 0, 1, 2: G, H, W of block `index` (chains in the order
+/* One block of the factorisation of dt (built first if needed; the unreduced chains' too, which
+ * no solve needs on reduced chains), copied to the host (synchronous).  which = 0, 1, 2: G, H, W of block `index` (chains in the order
  * (m index, class), blocks l = m .. L inside a chain; Nr x Nr complex row-major, 2 Nr^2
  * doubles): the twisted block Thomas factors of Sec. 3.2 with G = D'^-1, H = D'^-1 A,
  * W = D'^-1 C above the middle block of a chain, G = E'^-1, H = E'^-1 C, W = E'^-1 A
@@ -190,7 +190,8 @@ rsc_status rsc_implicit_solve(rsc_ctx* ctx, const double* rhs, double* x, double
  * (hi + lo, about 2^-48 relative).  For checks of the factorisation.                */
 rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, double* out_host);
 
-/* Wall time (s) of the context's last factorisation and whether it ran on the GPU. */
+/* Wall time (s) of the context's last factorisation and whether it ran on the GPU: the temperature
+ * operators and, where a solve needs them, the unreduced chains.                           */
 rsc_status rsc_factor_time(const rsc_ctx* ctx, double* seconds, int* on_gpu);
 /* The same for the context's last factorisation of the odd-even reduced chains
  * (rsc_tuning chain_cr; 0 s until one has run).                                  */
@@ -426,7 +427,9 @@ typedef struct {
                               computed on first use, on the GPU where factor_gpu puts
                               the FP64 factorisation (chain_parts = 1 and implicit
                               Coriolis only).  Default 1 on a mixed context; 0 = the
-                              unreduced chains.  Changes the order of the arithmetic.   */
+                              unreduced chains.  Changes the order of the arithmetic.
+                              (FP64 solves run on reduced chains wherever chain_parts = 1,
+                              the Coriolis term is implicit and their factors fit.)     */
   double ms[6];            /* after rsc_autotune: best times (ms) of products +
                               analysis (mixed), FP64 synthesis, RHS (mixed), FP64 chain
                               solve, double-float chain solve (0 if none ran); zero

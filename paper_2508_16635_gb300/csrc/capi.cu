@@ -27,6 +27,7 @@
 #include "krylov_split.cuh"
 #include "chain_df.cuh"
 #include "chain_cr.cuh"
+#include "chain_cr64.cuh"
 #include "products_sym.cuh"
 #include "radial_rhs_f32.cuh"
 #include "radial_rhs_par.cuh"
@@ -73,6 +74,8 @@ struct DevFactor {
   float4* Gr = nullptr;
   float4* Hr = nullptr;
   float4* Wr = nullptr;
+  double2 *D64 = nullptr, *G64 = nullptr, *H64 = nullptr, *W64 = nullptr;   // the same in FP64
+  bool cr_no_room = false;   // they did not fit: the FP64 solve runs on the unreduced chains
   double cr_s = 0.0;   // wall time of their factorisation (s)
   int cr_on_gpu = 0;   // where it ran
   bool valid = false;
@@ -156,6 +159,7 @@ struct rsc_ctx {
   float2* d_E01 = nullptr;     // E0, then E1, [j][k] {hi, lo} at the collocation radii
   double2* d_rowf64 = nullptr;    // [j] {2 / r^3, 2 / r^2}
   CrPair* d_pairf64 = nullptr;    // [p] {a l, a, c (l + 1), c}
+  double2* d_E01_64 = nullptr;    // [j][k] {E0, E1}
   float4* d_cr_rowf = nullptr;    // [j] {2 / r^3 hi, lo, 2 / r^2 hi, lo}
   float4* d_cr_pairf = nullptr;   // [p][2] {a l, a}, {c (l + 1), c} (coupling coefficients)
   float4* cr_w = nullptr;      // E0 u, E1 u of the odd blocks, [2][2 P Nr]
@@ -336,9 +340,26 @@ void free_factor(DevFactor& f) {
   cudaFree(f.Hs);
   cudaFree(f.Ws);
   void* extra[] = {f.parts, f.Vsp, f.Wsp, f.red, f.red_off, f.red_nu, f.zoff, f.unk_row, f.blk_z,
-                   f.zbuf, f.cr_odd_off, f.cr_red_off, f.Ds, f.Gr, f.Hr, f.Wr};
+                   f.zbuf, f.cr_odd_off, f.cr_red_off, f.Ds, f.Gr, f.Hr, f.Wr, f.D64, f.G64, f.H64, f.W64};
   for (void* b : extra) cudaFree(b);
   f = DevFactor();
+}
+
+// The parts of a slot that are added on first use, released when their factorisation fails (so that
+// the next use reports the failure again).
+void free_reduced(DevFactor& f) {
+  void* bufs[] = {f.cr_odd_off, f.cr_red_off, f.Ds, f.Gr, f.Hr, f.Wr, f.D64, f.G64, f.H64, f.W64};
+  for (void* b : bufs) cudaFree(b);
+  f.cr_odd_off = f.cr_red_off = nullptr;
+  f.Ds = f.Gr = f.Hr = f.Wr = nullptr;
+  f.D64 = f.G64 = f.H64 = f.W64 = nullptr;
+}
+void free_unreduced(DevFactor& f) {
+  void* bufs[] = {f.chain_off, f.G, f.H, f.W, f.Gs, f.Hs, f.Ws};
+  for (void* b : bufs) cudaFree(b);
+  f.chain_off = nullptr;
+  f.G = f.H = f.W = nullptr;
+  f.Gs = f.Hs = f.Ws = nullptr;
 }
 
 // Factorisations of one operator shared by several contexts (the instances of a batch with
@@ -704,7 +725,21 @@ bool factor_on_device(const rsc_ctx* ctx) {
   return ctx->factor_gpu && ctx->d.Nr <= kFacMaxNr && ctx->chain_parts == 1;
 }
 
-// The factors of one dt on the device (factor_gpu.cuh), FP64, and their double-float
+// The FP64 solve runs on odd-even reduced chains (chain_cr.cuh): wherever the chains are whole and
+// coupled.
+bool cr64_wanted(const rsc_ctx* ctx) { return ctx->chain_parts == 1 && !ctx->p.explicit_coriolis; }
+// The double-float solve of the mixed path does too (rsc_tuning chain_cr).
+bool cr_wanted(const rsc_ctx* ctx) {
+  return ctx->p.precision == RSC_MIXED && ctx->chain_cr && cr64_wanted(ctx);
+}
+// The factors of the unreduced chains are needed.
+bool full_wanted(const rsc_ctx* ctx) {
+  return !cr64_wanted(ctx) || (ctx->p.precision == RSC_MIXED && !ctx->chain_cr);
+}
+
+FacGeom fac_geom(const rsc_ctx* ctx, double dt);
+
+// The chain factors of one dt on the device (factor_gpu.cuh), FP64, and their double-float
 // copies on a mixed-precision context.
 rsc_status gpu_factor(rsc_ctx* ctx, double dt, DevFactor& f) {
   const Dims& d = ctx->d;
@@ -722,40 +757,24 @@ rsc_status gpu_factor(rsc_ctx* ctx, double dt, DevFactor& f) {
   CK(cudaMalloc(&f.G, nent * sizeof(double2)));
   CK(cudaMalloc(&f.H, nent * sizeof(double2)));
   CK(cudaMalloc(&f.W, nent * sizeof(double2)));
-  CK(cudaMalloc(&f.Tinv, (size_t)(d.L + 1) * blk * sizeof(double)));
   CK(cudaMemsetAsync(f.H, 0, nent * sizeof(double2), ctx->s));   // H of the end blocks stays 0
   CK(cudaMemsetAsync(f.W, 0, nent * sizeof(double2), ctx->s));
   int* status = nullptr;
-  CK(cudaMalloc(&status, (nchains + 1) * sizeof(int)));
-  CK(cudaMemsetAsync(status, 0, (nchains + 1) * sizeof(int), ctx->s));
-  FacGeom g;
-  g.Nr = d.Nr;
-  g.L = d.L;
-  g.nm = d.nm;
-  g.m_of = ctx->d_m_of;
+  CK(cudaMalloc(&status, nchains * sizeof(int)));
+  CK(cudaMemsetAsync(status, 0, nchains * sizeof(int), ctx->s));
+  FacGeom g = fac_geom(ctx, dt);
   g.chain_off = f.chain_off;
-  g.rc = ctx->d_rc;
-  g.E0 = ctx->d_Ef[0];
-  g.E1 = ctx->d_Ef[1];
-  g.E2 = ctx->d_Ef[2];
-  g.E4 = ctx->d_Ef[3];
-  g.Ek = ctx->p.Ek;
-  g.Pr = ctx->p.Pr;
-  g.inv_dt = std::isfinite(dt) ? 1.0 / dt : 0.0;
-  g.explicit_coriolis = ctx->p.explicit_coriolis ? 1 : 0;
   const size_t smem = fac_smem_bytes(d.Nr);
-  for (const void* fn : {(const void*)k_factor_half, (const void*)k_factor_mid, (const void*)k_factor_temp})
+  for (const void* fn : {(const void*)k_factor_half, (const void*)k_factor_mid})
     CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   double2* G = reinterpret_cast<double2*>(f.G);
   double2* H = reinterpret_cast<double2*>(f.H);
   double2* W = reinterpret_cast<double2*>(f.W);
-  k_factor_temp<<<d.L + 1, kFacThreads, smem, ctx->s>>>(g, f.Tinv, status + nchains);
-  CK(cudaGetLastError());
   k_factor_half<<<2 * nchains, kFacThreads, smem, ctx->s>>>(g, G, H, W, status);
   CK(cudaGetLastError());
   k_factor_mid<<<nchains, kFacThreads, smem, ctx->s>>>(g, G, H, W, status);
   CK(cudaGetLastError());
-  ctx->launches += 3;
+  ctx->launches += 2;
   if (ctx->p.precision == RSC_MIXED) {
     CK(cudaMalloc(&f.Gs, nent * sizeof(float4)));
     CK(cudaMalloc(&f.Hs, nent * sizeof(float4)));
@@ -767,16 +786,38 @@ rsc_status gpu_factor(rsc_ctx* ctx, double dt, DevFactor& f) {
     CK(cudaGetLastError());
     ctx->launches += 3;
   }
-  std::vector<int> hs(nchains + 1);
+  std::vector<int> hs(nchains);
   CK(cudaMemcpyAsync(hs.data(), status, hs.size() * sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
   CK(cudaStreamSynchronize(ctx->s));
   cudaFree(status);
-  for (int c = 0; c <= nchains; ++c)
+  for (int c = 0; c < nchains; ++c)
     if (hs[c]) {
-      ctx->err = c < nchains ? "singular block in the implicit operator (chain " + std::to_string(c) + ")"
-                             : std::string("singular temperature block");
+      ctx->err = "singular block in the implicit operator (chain " + std::to_string(c) + ")";
       return RSC_ESINGULAR;
     }
+  return RSC_OK;
+}
+
+// The temperature inverses of one dt on the device.
+rsc_status gpu_factor_temp(rsc_ctx* ctx, double dt, DevFactor& f) {
+  const Dims& d = ctx->d;
+  int* status = nullptr;
+  int bad = 0;
+  CK(cudaMalloc(&f.Tinv, (size_t)(d.L + 1) * d.Nr * d.Nr * sizeof(double)));
+  CK(cudaMalloc(&status, sizeof(int)));
+  CK(cudaMemsetAsync(status, 0, sizeof(int), ctx->s));
+  const size_t smem = fac_smem_bytes(d.Nr);
+  CK(cudaFuncSetAttribute((const void*)k_factor_temp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_factor_temp<<<d.L + 1, kFacThreads, smem, ctx->s>>>(fac_geom(ctx, dt), f.Tinv, status);
+  CK(cudaGetLastError());
+  ctx->launches += 1;
+  CK(cudaMemcpyAsync(&bad, status, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+  CK(cudaStreamSynchronize(ctx->s));
+  cudaFree(status);
+  if (bad) {
+    ctx->err = "singular temperature block";
+    return RSC_ESINGULAR;
+  }
   return RSC_OK;
 }
 
@@ -785,7 +826,9 @@ rsc_status gpu_factor(rsc_ctx* ctx, double dt, DevFactor& f) {
 rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
   const auto t_fac0 = std::chrono::steady_clock::now();
   if (factor_on_device(ctx)) {
-    CKS(gpu_factor(ctx, dt, f));
+    // the unreduced chains' factors only where something solves with them (else on first use)
+    CKS(gpu_factor_temp(ctx, dt, f));
+    if (full_wanted(ctx)) CKS(gpu_factor(ctx, dt, f));
     ctx->factor_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_fac0).count();
     ctx->factor_on_gpu = 1;
     f.dt = dt;
@@ -854,12 +897,6 @@ rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
   return RSC_OK;
 }
 
-
-// The double-float solve runs on odd-even reduced chains (chain_cr.cuh) on this context.
-bool cr_wanted(const rsc_ctx* ctx) {
-  return ctx->p.precision == RSC_MIXED && ctx->chain_cr && ctx->chain_parts == 1 &&
-         !ctx->p.explicit_coriolis;
-}
 
 // Double-float copy of complex FP64 blocks: hi = the entry rounded to FP32, lo = the
 // remainder rounded to FP32.
@@ -952,7 +989,7 @@ rsc_status gpu_factor_cr(rsc_ctx* ctx, DevFactor* f) {
   float4** dsts[] = {&f->Ds, &f->Gr, &f->Hr, &f->Wr};
   const double2* srcs[] = {Di, G, H, W};
   const size_t ns[] = {eo, er, er, er};
-  for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+  for (int q = 0; q < 4 && ctx->p.precision == RSC_MIXED && e == cudaSuccess; ++q) {
     ok(cudaMalloc(dsts[q], ns[q] * sizeof(float4)));
     if (e != cudaSuccess) break;
     const int nbk = (int)std::min<size_t>((ns[q] + 255) / 256, 152 * 32);
@@ -963,6 +1000,11 @@ rsc_status gpu_factor_cr(rsc_ctx* ctx, DevFactor* f) {
   if (e == cudaSuccess)
     ok(cudaMemcpyAsync(hs.data(), status, nchains * sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
   ok(cudaStreamSynchronize(ctx->s));
+  f->D64 = Di;
+  f->G64 = G;
+  f->H64 = H;
+  f->W64 = W;
+  Di = G = H = W = nullptr;
   release();
   ctx->launches += 8;
   if (e != cudaSuccess) {
@@ -999,6 +1041,9 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
       e[i] = make_float2(ah, (float)(a - (double)ah));
     }
     CKS(upload(ctx, &ctx->d_E01, e.data(), e.size()));
+    std::vector<double2> e64((size_t)d.Nr * d.Nr);
+    for (size_t i = 0; i < e64.size(); ++i) e64[i] = make_double2(ctx->t.Ec[0][i], ctx->t.Ec[1][i]);
+    CKS(upload(ctx, &ctx->d_E01_64, e64.data(), e64.size()));
     auto pair_of = [](double a, double b) {
       const float ah = (float)a, bh = (float)b;
       return make_float4(ah, (float)(a - (double)ah), bh, (float)(b - (double)bh));
@@ -1019,10 +1064,14 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
     CKS(upload(ctx, &ctx->d_cr_pairf, pairf.data(), pairf.size()));
     CK(cudaMalloc(&ctx->cr_w, (size_t)2 * 2 * d.P * d.Nr * sizeof(float4)));
   }
-  if (f->Ds) return RSC_OK;
+  if (f->D64) return RSC_OK;
   const auto t0 = std::chrono::steady_clock::now();
   if (factor_on_device(ctx)) {
-    CKS(gpu_factor_cr(ctx, f));
+    const rsc_status st = gpu_factor_cr(ctx, f);
+    if (st != RSC_OK) {
+      free_reduced(*f);
+      return st;
+    }
     f->cr_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     f->cr_on_gpu = 1;
     ctx->factor_cr_s = f->cr_s;
@@ -1035,12 +1084,19 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
     ctx->err = "singular block in the reduced implicit operator (chain " + std::to_string(bad - 1) + ")";
     return RSC_ESINGULAR;
   }
-  CKS(upload(ctx, &f->cr_odd_off, hc.odd_off.data(), hc.odd_off.size()));
-  CKS(upload(ctx, &f->cr_red_off, hc.red_off.data(), hc.red_off.size()));
-  CKS(upload_split(ctx, hc.Dinv, &f->Ds));
-  CKS(upload_split(ctx, hc.G, &f->Gr));
-  CKS(upload_split(ctx, hc.H, &f->Hr));
-  CKS(upload_split(ctx, hc.W, &f->Wr));
+  rsc_status st = upload(ctx, &f->cr_odd_off, hc.odd_off.data(), hc.odd_off.size());
+  if (st == RSC_OK) st = upload(ctx, &f->cr_red_off, hc.red_off.data(), hc.red_off.size());
+  const std::vector<cplx>* src[] = {&hc.Dinv, &hc.G, &hc.H, &hc.W};
+  double2** dst[] = {&f->D64, &f->G64, &f->H64, &f->W64};
+  float4** dsf[] = {&f->Ds, &f->Gr, &f->Hr, &f->Wr};
+  for (int q = 0; q < 4 && st == RSC_OK; ++q) {
+    st = upload(ctx, dst[q], reinterpret_cast<const double2*>(src[q]->data()), src[q]->size());
+    if (st == RSC_OK && ctx->p.precision == RSC_MIXED) st = upload_split(ctx, *src[q], dsf[q]);
+  }
+  if (st != RSC_OK) {
+    free_reduced(*f);
+    return st;
+  }
   f->cr_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   f->cr_on_gpu = 0;
   ctx->factor_cr_s = f->cr_s;
@@ -1054,12 +1110,31 @@ rsc_status ensure_cr_locked(rsc_ctx* ctx, DevFactor* f) {
   return ensure_cr(ctx, f);
 }
 
+// The factors of the unreduced chains, if f has none yet.
+rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
+  std::unique_lock<std::mutex> lock;
+  if (ctx->share) lock = std::unique_lock<std::mutex>(ctx->share->mu);
+  if (f->G) return RSC_OK;
+  const rsc_status st = gpu_factor(ctx, f->dt, *f);
+  if (st != RSC_OK) free_unreduced(*f);
+  return st;
+}
+
 rsc_status get_factor_slot(rsc_ctx* ctx, double dt, DevFactor** out);
 
 // A shared slot gains its reduced factors under the share's lock.
 rsc_status get_factor(rsc_ctx* ctx, double dt, DevFactor** out) {
   CKS(get_factor_slot(ctx, dt, out));
-  return cr_wanted(ctx) ? ensure_cr_locked(ctx, *out) : RSC_OK;
+  DevFactor* f = *out;
+  if (full_wanted(ctx)) CKS(ensure_full(ctx, f));
+  if (!cr64_wanted(ctx) || (f->cr_no_room && !cr_wanted(ctx))) return RSC_OK;
+  const rsc_status st = ensure_cr_locked(ctx, f);
+  if (st != RSC_ENOMEM || cr_wanted(ctx)) return st;
+  // no room for the reduced factorisation (its scratch takes half as much again as the unreduced
+  // factors): the FP64 solve on the unreduced chains
+  cudaGetLastError();
+  f->cr_no_room = true;
+  return ensure_full(ctx, f);
 }
 
 rsc_status get_factor_slot(rsc_ctx* ctx, double dt, DevFactor** out) {
@@ -1329,8 +1404,15 @@ size_t chain_smem_async(const Dims& d, int CS, bool outward, int NS) {
              sizeof(double2) + 16;
 }
 
+// The blocks of the FP64 sweeps: the full chains, or the odd-even reduced ones (every second block).
+struct ChainBlocks {
+  const long* off;
+  const double2 *H, *W;
+  int bs;
+};
+
 template <int Q, int NS>
-cudaError_t launch_chain_async_q(rsc_ctx* ctx, const DevFactor* f, double* out, bool outward) {
+cudaError_t launch_chain_async_q(rsc_ctx* ctx, const ChainBlocks& cb, double* out, bool outward) {
   const Dims& d = ctx->d;
   const int CS = ctx->cluster;
   const int RPC = (d.Nr + CS - 1) / CS;
@@ -1348,20 +1430,18 @@ cudaError_t launch_chain_async_q(rsc_ctx* ctx, const DevFactor* f, double* out, 
   cfg.numAttrs = 1;
   const int cap = chain_steps_cap(d);
   if (outward)
-    return cudaLaunchKernelEx(&cfg, k_chain_out_async<Q / NS, NS>, ctx->geom(),
-                              (const long*)f->chain_off, (const double2*)f->H,
-                              (const double2*)f->W, reinterpret_cast<double2*>(out),
-                              (const double2*)ctx->mid, CS, cap, ctx->d_status);
-  return cudaLaunchKernelEx(&cfg, k_chain_half_async<Q / NS, NS>, ctx->geom(),
-                            (const long*)f->chain_off, (const double2*)f->H,
-                            reinterpret_cast<double2*>(out), ctx->mid, CS, cap, ctx->d_status);
+    return cudaLaunchKernelEx(&cfg, k_chain_out_async<Q / NS, NS>, ctx->geom(), cb.off, cb.H, cb.W,
+                              reinterpret_cast<double2*>(out), (const double2*)ctx->mid, CS, cap,
+                              ctx->d_status, cb.bs);
+  return cudaLaunchKernelEx(&cfg, k_chain_half_async<Q / NS, NS>, ctx->geom(), cb.off, cb.H,
+                            reinterpret_cast<double2*>(out), ctx->mid, CS, cap, ctx->d_status, cb.bs);
 }
 
 template <int Q>
-cudaError_t launch_chain_q(rsc_ctx* ctx, const DevFactor* f, double* out, bool outward) {
-  if (ctx->chain_async == 1) return launch_chain_async_q<Q, 2>(ctx, f, out, outward);
+cudaError_t launch_chain_q(rsc_ctx* ctx, const ChainBlocks& cb, double* out, bool outward) {
+  if (ctx->chain_async == 1) return launch_chain_async_q<Q, 2>(ctx, cb, out, outward);
   if (ctx->chain_async == 2) {
-    if constexpr (Q % 4 == 0) return launch_chain_async_q<Q, 4>(ctx, f, out, outward);
+    if constexpr (Q % 4 == 0) return launch_chain_async_q<Q, 4>(ctx, cb, out, outward);
     return cudaErrorInvalidValue;
   }
   const Dims& d = ctx->d;
@@ -1380,20 +1460,21 @@ cudaError_t launch_chain_q(rsc_ctx* ctx, const DevFactor* f, double* out, bool o
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (outward)
-    return cudaLaunchKernelEx(&cfg, k_chain_out<Q>, ctx->geom(), (const long*)f->chain_off,
-                              (const double2*)f->H, (const double2*)f->W,
-                              reinterpret_cast<double2*>(out), (const double2*)ctx->mid, CS);
-  return cudaLaunchKernelEx(&cfg, k_chain_half<Q>, ctx->geom(), (const long*)f->chain_off,
-                            (const double2*)f->H, reinterpret_cast<double2*>(out), ctx->mid, CS);
+    return cudaLaunchKernelEx(&cfg, k_chain_out<Q>, ctx->geom(), cb.off, cb.H, cb.W,
+                              reinterpret_cast<double2*>(out), (const double2*)ctx->mid, CS, cb.bs);
+  return cudaLaunchKernelEx(&cfg, k_chain_half<Q>, ctx->geom(), cb.off, cb.H,
+                            reinterpret_cast<double2*>(out), ctx->mid, CS, cb.bs);
 }
 
-cudaError_t launch_chain(rsc_ctx* ctx, const DevFactor* f, double* out, bool outward) {
+cudaError_t launch_chain(rsc_ctx* ctx, const DevFactor* f, double* out, bool outward, bool cr) {
+  const ChainBlocks cb = cr ? ChainBlocks{f->cr_red_off, f->H64, f->W64, 2}
+                            : ChainBlocks{f->chain_off, f->H, f->W, 1};
   switch (chain_maxq(ctx->d.Nr)) {
-    case 2: return launch_chain_q<2>(ctx, f, out, outward);
-    case 4: return launch_chain_q<4>(ctx, f, out, outward);
-    case 8: return launch_chain_q<8>(ctx, f, out, outward);
-    case 12: return launch_chain_q<12>(ctx, f, out, outward);
-    default: return launch_chain_q<16>(ctx, f, out, outward);
+    case 2: return launch_chain_q<2>(ctx, cb, out, outward);
+    case 4: return launch_chain_q<4>(ctx, cb, out, outward);
+    case 8: return launch_chain_q<8>(ctx, cb, out, outward);
+    case 12: return launch_chain_q<12>(ctx, cb, out, outward);
+    default: return launch_chain_q<16>(ctx, cb, out, outward);
   }
 }
 
@@ -1478,9 +1559,32 @@ void launch_cr_pass_df(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) 
         ctx->rhs, o);
 }
 
-void launch_cr_pass(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
+void launch_cr_pass_64(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
+  const Dims& d = ctx->d;
+  const size_t v = (size_t)d.Nr * sizeof(double2);
+  const int* odd = ctx->d_cr_pairs;
+  const int* even = ctx->d_cr_pairs + ctx->n_cr_odd;
+  double2 *o = reinterpret_cast<double2*>(out), *w = reinterpret_cast<double2*>(ctx->cr_w);
+  const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));   // as launch_cr_pass_df
+  if (pass == 0)
+    k_cr_odd<<<2 * ctx->n_cr_odd, thr, 2 * v, ctx->s>>>(ctx->geom(), odd, f->cr_odd_off, f->D64,
+                                                        ctx->d_E01_64, ctx->rhs, w);
+  else if (pass == 1)
+    k_cr_even<<<2 * ctx->n_cr_even, thr, v, ctx->s>>>(ctx->geom(), even, f->cr_red_off, f->G64,
+                                                      ctx->d_rowf64, ctx->d_pairf64, ctx->rhs, w, o);
+  else
+    k_cr_back<<<2 * ctx->n_cr_odd, thr, 4 * v, ctx->s>>>(ctx->geom(), odd, f->cr_odd_off, f->D64,
+                                                         ctx->d_E01_64, ctx->d_rowf64, ctx->d_pairf64,
+                                                         ctx->rhs, o);
+}
+
+void launch_cr_pass(rsc_ctx* ctx, const DevFactor* f, double* out, int pass, bool df) {
   const int n = 2 * (pass == 1 ? ctx->n_cr_even : ctx->n_cr_odd);
   if (n == 0) return;
+  if (!df) {
+    launch_cr_pass_64(ctx, f, out, pass);
+    return;
+  }
   // five CTAs per SM where all are resident at once that way only (chain_cr.cuh)
   if (n > 4 * ctx->nsm && n <= 5 * ctx->nsm)
     launch_cr_pass_df<5>(ctx, f, out, pass);
@@ -1505,8 +1609,8 @@ void launch_gemv_df(rsc_ctx* ctx, const DevFactor* f, double* out) {
 // and chain_df is on); otherwise the FP64 kernels.
 rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = false,
                        bool temp = true) {
-  df = df && f->Gs && f->Hs && f->Ws && ctx->chain_df != 0;
-  const bool cr = df && cr_wanted(ctx) && f->Ds && ctx->d_E01;
+  df = df && ctx->p.precision == RSC_MIXED && ctx->chain_df != 0;
+  const bool cr = df ? cr_wanted(ctx) : cr64_wanted(ctx) && f->D64;
   const Dims& d = ctx->d;
   // the temperature solve depends only on the right-hand side: it runs on a second stream
   // beside the e/f chain solve (sequentially while tracing, so that every launch is timed)
@@ -1533,22 +1637,22 @@ rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = 
     {
       KSpan sp(ctx, RSC_K_CHAIN_RED, bo * nr2 * 16.0 + bo * d.Nr * 16.0 * 3.0 + tab,
                bo * nr2 * 8.0 + bo * nr2 * 4.0);
-      launch_cr_pass(ctx, f, out, 0);
+      launch_cr_pass(ctx, f, out, 0, df);
       CK(cudaGetLastError());
     }
     {
       KSpan sp(ctx, RSC_K_CHAIN_RED, be * nr2 * 16.0 + be * d.Nr * 16.0 * 6.0, be * nr2 * 8.0);
-      launch_cr_pass(ctx, f, out, 1);
+      launch_cr_pass(ctx, f, out, 1, df);
       CK(cudaGetLastError());
     }
     for (int outward = 0; outward < 2; ++outward) {
       KSpan sp(ctx, RSC_K_CHAIN_SEQ, be * nr2 * 16.0 + 2.0 * be * d.Nr * 16.0, be * nr2 * 8.0);
-      CK(launch_chain_df(ctx, f, out, outward != 0, true));
+      CK(df ? launch_chain_df(ctx, f, out, outward != 0, true) : launch_chain(ctx, f, out, outward != 0, true));
     }
     {
       KSpan sp(ctx, RSC_K_CHAIN_RED, bo * nr2 * 16.0 + bo * d.Nr * 16.0 * 4.0 + tab,
                bo * nr2 * 8.0 + bo * nr2 * 4.0);
-      launch_cr_pass(ctx, f, out, 2);
+      launch_cr_pass(ctx, f, out, 2, df);
       CK(cudaGetLastError());
     }
   }
@@ -1566,12 +1670,12 @@ rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = 
     // forward half-sweeps read H of about half the blocks each way, outward sweeps W
     KSpan sp(ctx, RSC_K_CHAIN_SEQ, 2.0 * d.P * d.Nr * d.Nr * 16.0 + 4.0 * d.P * d.Nr * 16.0,
              2.0 * d.P * d.Nr * d.Nr * 8.0);
-    CK(df ? launch_chain_df(ctx, f, out, false) : launch_chain(ctx, f, out, false));
+    CK(df ? launch_chain_df(ctx, f, out, false) : launch_chain(ctx, f, out, false, false));
   }
   if (!cr && !ctx->p.explicit_coriolis) {
     KSpan sp(ctx, RSC_K_CHAIN_SEQ, 2.0 * d.P * d.Nr * d.Nr * 16.0 + 4.0 * d.P * d.Nr * 16.0,
              2.0 * d.P * d.Nr * d.Nr * 8.0);
-    CK(df ? launch_chain_df(ctx, f, out, true) : launch_chain(ctx, f, out, true));
+    CK(df ? launch_chain_df(ctx, f, out, true) : launch_chain(ctx, f, out, true, false));
   }
   if (df && f->npart && !ctx->p.explicit_coriolis) {
     // partitioned chains: reduced systems, then the correction of every part
@@ -2509,12 +2613,13 @@ rsc_status autotune(rsc_ctx* ctx, rsc_tuning* out) {
     ctx->chain_async = ba;
     ctx->tune_ms[3] = best;
     // mixed path: the double-float chain solve against the best FP64 one
-    if (st == RSC_OK && f->Gs) {
+    if (st == RSC_OK && ctx->p.precision == RSC_MIXED) {
       double best_df = 1e30;
       int bn = 0, bcs = t.chain_df_cluster, bcr = 0;
       const int saved_cr = ctx->chain_cr;
       for (int cr : {0, 1}) {   // the unreduced chains, then the odd-even reduced ones
         ctx->chain_cr = cr;
+        if (!cr && st == RSC_OK) st = ensure_full(ctx, f);
         if (cr && (st != RSC_OK || !cr_wanted(ctx))) break;
         if (cr) st = ensure_cr_locked(ctx, f);
         for (int ns : {2, 4}) {
@@ -2769,7 +2874,7 @@ rsc_status rsc_destroy(rsc_ctx* ctx) {
   if (ctx->s2) cudaStreamSynchronize(ctx->s2), cudaStreamDestroy(ctx->s2);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_EcT4, ctx->res_z, ctx->d_rowf64, ctx->d_pairf64, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
+  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_EcT4, ctx->res_z, ctx->d_rowf64, ctx->d_pairf64, ctx->d_E01_64, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
                   ctx->d_rc, ctx->d_rd, ctx->d_EcT0, ctx->d_EcT2, ctx->d_EdT0, ctx->d_EdT1,
                   ctx->d_EdT2, ctx->d_R0T, ctx->d_R1T, ctx->f_EdT0, ctx->f_EdT1,
                   ctx->f_EdT2, ctx->f_R0T, ctx->f_R1T, ctx->f_rd, ctx->f_EcT0, ctx->f_EcT2, ctx->SR, ctx->FC, ctx->FCU, ctx->UG, ctx->FA,
@@ -3065,6 +3170,7 @@ rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, doub
     }
     return RSC_OK;
   }
+  if (which < 3) CKS(ensure_full(ctx, f));
   if (which == 3)
     CK(cudaMemcpyAsync(out_host, f->Tinv + index * blk, blk * sizeof(double),
                        cudaMemcpyDeviceToHost, ctx->s));

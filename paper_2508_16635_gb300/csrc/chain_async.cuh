@@ -6,6 +6,8 @@
 //   * a block's new rows travel to every CTA of the cluster as st.async stores that
 //     complete on the receiver's mbarrier (expect_tx of Nr x 16 bytes per step), instead of
 //     a cluster-wide barrier per block.
+// bs = 2 sweeps every second block (the reduced chains of chain_cr64.cuh, chain_off their first blocks in
+// H and W), 1 the full chains.
 // Every wait on an mbarrier is bounded; a timeout sets *status = RSC_ETIMEOUT (7) and the
 // sweep runs on (with meaningless values) so that no peer waits forever; the kernel ends
 // with a hardware cluster barrier so no CTA leaves while peers may still write into it.
@@ -120,11 +122,11 @@ template <int QH, int NS>
 __global__ void k_chain_half_async(DevGeom g, const long* __restrict__ chain_off,
                                    const double2* __restrict__ H, double2* __restrict__ out,
                                    double2* __restrict__ mid, int CS, int steps_cap,
-                                   int* __restrict__ status) {
+                                   int* __restrict__ status, int bs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 ca_sh[];
-  const ChainInfo ci = chain_info(g, chain_off, CS);
+  const ChainInfo ci = chain_info(g, chain_off, CS, bs);
   const int Nr = ci.Nr;
   const CaLane c = ca_lane<QH, NS>(Nr, CS, (int)cluster.block_rank());
   double2* v = ca_sh;                       // [2][Nr]
@@ -202,11 +204,11 @@ template <int QH, int NS>
 __global__ void k_chain_out_async(DevGeom g, const long* __restrict__ chain_off,
                                   const double2* __restrict__ H, const double2* __restrict__ W,
                                   double2* __restrict__ out, const double2* __restrict__ mid,
-                                  int CS, int steps_cap, int* __restrict__ status) {
+                                  int CS, int steps_cap, int* __restrict__ status, int bs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 ca_sh[];
-  const ChainInfo ci = chain_info(g, chain_off, CS);
+  const ChainInfo ci = chain_info(g, chain_off, CS, bs);
   const int Nr = ci.Nr;
   const CaLane c = ca_lane<QH, NS>(Nr, CS, (int)cluster.block_rank());
   double2* v = ca_sh;

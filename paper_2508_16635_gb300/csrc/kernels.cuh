@@ -673,11 +673,11 @@ __device__ __forceinline__ ChainInfo chain_info(const DevGeom& g, const long* ch
 template <int MAXQ>
 __global__ void k_chain_half(DevGeom g, const long* __restrict__ chain_off,
                              const double2* __restrict__ H, double2* __restrict__ out,
-                             double2* __restrict__ mid, int CS) {
+                             double2* __restrict__ mid, int CS, int bs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 sv[];  // [2][Nr] ping-pong, then hist[steps][RPC]
-  const ChainInfo ci = chain_info(g, chain_off, CS);
+  const ChainInfo ci = chain_info(g, chain_off, CS, bs);
   const int Nr = ci.Nr;
   const int rank = (int)cluster.block_rank();
   const int RPC = (Nr + CS - 1) / CS;
@@ -740,11 +740,11 @@ __global__ void k_chain_half(DevGeom g, const long* __restrict__ chain_off,
 template <int MAXQ>
 __global__ void k_chain_out(DevGeom g, const long* __restrict__ chain_off,
                             const double2* __restrict__ H, const double2* __restrict__ W,
-                            double2* __restrict__ out, const double2* __restrict__ mid, int CS) {
+                            double2* __restrict__ out, const double2* __restrict__ mid, int CS, int bs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 sv[];  // [2][Nr] ping-pong, [2][Nr] middle inputs, hist[steps][RPC]
-  const ChainInfo ci = chain_info(g, chain_off, CS);
+  const ChainInfo ci = chain_info(g, chain_off, CS, bs);
   const int Nr = ci.Nr;
   const int rank = (int)cluster.block_rank();
   const int RPC = (Nr + CS - 1) / CS;

@@ -112,17 +112,17 @@ def test_radial_stages_by_reflection(torch, L, Ms, Nr):
 # test_implicit_solve_backward_error_* of test_gpu_parity.py.
 @pytest.mark.parametrize("L,Ms,Nr", [(4, 4, 6), (9, 3, 17), (12, 5, 33), (7, 7, 64), (8, 8, 65),
                                      (5, 4, 128), (34, 1, 8)])
-@pytest.mark.parametrize("precision", ["mixed"])
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_reduced_chain_passes(torch, L, Ms, Nr, precision):
     from paper_2508_16635_gb300 import RotatingShell
-    from tests.test_gpu_parity import U48, _random_rhs, _solve_errors
+    from tests.test_gpu_parity import U48, U64, _random_rhs, _solve_errors
     s = Shell(L, Ms, Nr, 1e-3, 80.0)
     gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0, precision=precision)
     b = _random_rhs(s, 41)
     x = gpu.implicit_solve(torch.tensor(s.to_real(b), device="cuda"), 2e-3).cpu().numpy()
     eta, fwd, fwd_T = _solve_errors(s, 2e-3, b, s.to_complex(x))
-    assert eta < 64 * U48
-    assert fwd < 32 * 1e-10
+    assert eta < 64 * (U48 if precision == "mixed" else U64)
+    assert fwd < (32 * 1e-10 if precision == "mixed" else 1e-11)
     assert fwd_T < 1e-12
     gpu.close()
 
