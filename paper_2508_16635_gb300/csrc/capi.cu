@@ -166,6 +166,8 @@ struct rsc_ctx {
   // second stream: the temperature solve runs beside the e/f chain solve
   cudaStream_t s2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  bool joined = false;      // the next launch follows work of the second stream
+  bool capturing = false;   // the stream is captured into a graph
   // radii per block of the CUDA-core FP32 analysis ([1]); the FP64 transforms have one shape and
   // carry their rsc_tuning fields only
   int rt_synth[2] = {1, 1}, rt_anal[2] = {1, 1};
@@ -267,6 +269,17 @@ cudaEvent_t take_event(rsc_ctx* ctx) {
   return e;
 }
 
+// The attribute of an early launch, or none behind work of the second stream (a full dependency) and
+// in a captured graph, whose edges are quicker without it (four FP64 actions at L = 127 4243 us
+// replayed without, 4324 us with).
+int early_attr(rsc_ctx* ctx, cudaLaunchAttribute* attr) {
+  const bool early = !ctx->joined && !ctx->capturing;
+  ctx->joined = false;
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
+  return early ? 1 : 0;
+}
+
 // Brackets one kernel launch: counts it, adds its algorithmic bytes / flops
 // and, when tracing is on, records CUDA events around it on the context stream.
 struct KSpan {
@@ -291,6 +304,21 @@ struct KSpan {
     }
   }
 };
+
+// Launch on the context's stream that may start before the kernel ahead of it has ended: for kernels
+// that begin with grid_begin() only.
+template <class... E, class... A>
+cudaError_t launch(rsc_ctx* ctx, void (*kernel)(E...), dim3 grid, dim3 block, size_t smem, A&&... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->s;
+  cudaLaunchAttribute attr[1];
+  cfg.attrs = attr;
+  cfg.numAttrs = early_attr(ctx, attr);
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);
+}
 
 void drain_events(rsc_ctx* ctx) {
   if (ctx->ev_pending.empty()) return;
@@ -1195,16 +1223,16 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
     const double2* xx = reinterpret_cast<const double2*>(x);
     float2* sr = reinterpret_cast<float2*>(ctx->SR);
     switch (radial_fixed(d)) {
-      case 1: k_radial_f32<64, 96><<<gr, bl, sm, ctx->s>>>(g, xx, sr); break;
-      case 2: k_radial_f32<96, 144><<<gr, bl, sm, ctx->s>>>(g, xx, sr); break;
-      default: k_radial_f32<0, 0><<<gr, bl, sm, ctx->s>>>(g, xx, sr); break;
+      case 1: launch(ctx, (k_radial_f32<64, 96>), gr, bl, sm, g, xx, sr); break;
+      case 2: launch(ctx, (k_radial_f32<96, 144>), gr, bl, sm, g, xx, sr); break;
+      default: launch(ctx, (k_radial_f32<0, 0>), gr, bl, sm, g, xx, sr); break;
     }
   } else if constexpr (sizeof(R) == 8) {
     const int ppb = par_pairs((d.Nd + 1) / 2), tw = par_task_threads((d.Nd + 1) / 2);
-    k_radial_par<<<(d.P + ppb - 1) / ppb, 2 * tw, radial_par_smem(d.Nr, d.Nd), ctx->s>>>(
+    launch(ctx, k_radial_par, (d.P + ppb - 1) / ppb, 2 * tw, radial_par_smem(d.Nr, d.Nd),
         g, par_tables(ctx), reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(ctx->SR), ppb);
   } else {
-    k_radial<R><<<d.P, round32(std::max(d.Nd, 32)), 3 * d.Nr * sizeof(V), ctx->s>>>(
+    launch(ctx, k_radial<R>, d.P, round32(std::max(d.Nd, 32)), 3 * d.Nr * sizeof(V),
         g, reinterpret_cast<const double2*>(x), reinterpret_cast<V*>(ctx->SR));
   }
   CK(cudaGetLastError());
@@ -1221,16 +1249,16 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
     const bool pipe = ctx->synth_pipe != 0;
     const size_t smem = tc_synth_smem(ctx->tc_kmax, pipe);
     if (pipe)
-      k_synth_tc<true><<<grid, kTcThreads, smem, ctx->s>>>(g, tt, reinterpret_cast<const float2*>(ctx->SR),
+      launch(ctx, k_synth_tc<true>, grid, kTcThreads, smem, g, tt, reinterpret_cast<const float2*>(ctx->SR),
                                                     reinterpret_cast<float2*>(FCout));
     else
-      k_synth_tc<false><<<grid, kTcThreads, smem, ctx->s>>>(g, tt, reinterpret_cast<const float2*>(ctx->SR),
+      launch(ctx, k_synth_tc<false>, grid, kTcThreads, smem, g, tt, reinterpret_cast<const float2*>(ctx->SR),
                                                      reinterpret_cast<float2*>(FCout));
     CK(cudaGetLastError());
   } else {
     const auto& sl = ctx->sl[0];
     const SlTables tt{sl.tiles, sl.off, sl.ea, sl.nt, sl.ks, ctx->d_status};
-    k_synth_sl<<<dim3((d.Nd + kSsRad - 1) / kSsRad, d.nm, sl.nt), kSsThreads, ss_smem(sl.ks, sl.nst), ctx->s>>>(
+    launch(ctx, k_synth_sl, dim3((d.Nd + kSsRad - 1) / kSsRad, d.nm, sl.nt), kSsThreads, ss_smem(sl.ks, sl.nst),
         g, tt, sl.nst, reinterpret_cast<const double2*>(ctx->SR), reinterpret_cast<double2*>(FCout));
     CK(cudaGetLastError());
   }
@@ -1275,7 +1303,7 @@ void launch_products(rsc_ctx* ctx, int mode, const ProdShape& ps, const void* fc
   V* fa = reinterpret_cast<V*>(ctx->FA);
   R* ug = reinterpret_cast<R*>(ctx->UG);
   auto go = [&](auto kernel) {
-    kernel<<<grid, ps.LT * ps.S, ps.smem, ctx->s>>>(g, T, (R)ctx->p.Ek, c, fa, ug, ps.LT, ps.S, ps.Q);
+    launch(ctx, kernel, grid, ps.LT * ps.S, ps.smem, g, T, (R)ctx->p.Ek, c, fa, ug, ps.LT, ps.S, ps.Q);
   };
   auto pick = [&](auto even, auto quads) {
     constexpr bool E = decltype(even)::value;
@@ -1316,16 +1344,15 @@ rsc_status stage_products_analysis(rsc_ctx* ctx, bool lin) {
   if constexpr (sizeof(R) == 8) {
     const auto& sl = ctx->sl[1];
     const SlTables ta{sl.tiles, sl.off, sl.ea, sl.nt, sl.ks, ctx->d_status};
-    k_analysis_sl<<<dim3((d.Nd + kSaRad - 1) / kSaRad, d.nm), kSaThreads, sa_smem(sl.ks, sl.nst), ctx->s>>>(
+    launch(ctx, k_analysis_sl, dim3((d.Nd + kSaRad - 1) / kSaRad, d.nm), kSaThreads, sa_smem(sl.ks, sl.nst),
         g, ta, sl.nst, reinterpret_cast<const double2*>(ctx->FA), reinterpret_cast<double2*>(ctx->AR));
   } else if (ctx->anal_tc) {
     TaTables ta{ctx->ta_tiles, ctx->ta_off, ctx->ta_nchunk, ctx->d_status};
-    k_analysis_tc<<<dim3(d.nm, (d.Nd + kTaRadii - 1) / kTaRadii), kTaThreads, ta_smem(), ctx->s>>>(
+    launch(ctx, k_analysis_tc, dim3(d.nm, (d.Nd + kTaRadii - 1) / kTaRadii), kTaThreads, ta_smem(),
         g, ta, reinterpret_cast<const float2*>(ctx->FA), reinterpret_cast<float2*>(ctx->AR));
   } else {
     const int RTa = ctx->rt_anal[1], TC = ctx->atc[1];
-    k_analysis<float><<<dim3(d.nm, (d.Nd + RTa - 1) / RTa), dim3(round32(d.L + 1), RTa),
-                        analysis_smem<float>(d, RTa, TC), ctx->s>>>(
+    launch(ctx, k_analysis<float>, dim3(d.nm, (d.Nd + RTa - 1) / RTa), dim3(round32(d.L + 1), RTa), analysis_smem<float>(d, RTa, TC),
         g, leg<float>(ctx).view(), reinterpret_cast<const float2*>(ctx->FA),
         reinterpret_cast<float2*>(ctx->AR), TC);
   }
@@ -1355,9 +1382,9 @@ rsc_status stage_rhs(rsc_ctx* ctx, const RhsParams& rp, const double* x, const d
       const double2* xx = reinterpret_cast<const double2*>(x);
       const double2* uu = reinterpret_cast<const double2*>(U);
       switch (radial_fixed(d)) {
-        case 1: k_rhs_lin<64, 96><<<gr, bl, sm, ctx->s>>>(g, rp, arp, xx, uu, u_orig, out); break;
-        case 2: k_rhs_lin<96, 144><<<gr, bl, sm, ctx->s>>>(g, rp, arp, xx, uu, u_orig, out); break;
-        default: k_rhs_lin<0, 0><<<gr, bl, sm, ctx->s>>>(g, rp, arp, xx, uu, u_orig, out); break;
+        case 1: launch(ctx, (k_rhs_lin<64, 96>), gr, bl, sm, g, rp, arp, xx, uu, u_orig, out); break;
+        case 2: launch(ctx, (k_rhs_lin<96, 144>), gr, bl, sm, g, rp, arp, xx, uu, u_orig, out); break;
+        default: launch(ctx, (k_rhs_lin<0, 0>), gr, bl, sm, g, rp, arp, xx, uu, u_orig, out); break;
       }
       CK(cudaGetLastError());
       return RSC_OK;
@@ -1367,14 +1394,13 @@ rsc_status stage_rhs(rsc_ctx* ctx, const RhsParams& rp, const double* x, const d
     // FP64 sums by reflection (k_rhs keeps the explicit Coriolis rows and FP32 Jacobian actions)
     const double* second = rp.mode == 3 ? (xe && xe != x ? xe : nullptr) : rp.J >= 0 ? U : nullptr;
     const int ppb = par_pairs((d.Nr + 1) / 2), tw = par_task_threads((d.Nr + 1) / 2);
-    k_rhs_par<R><<<(d.P + ppb - 1) / ppb, (second ? 6 : 4) * tw,
-                   rhs_par_smem(d.Nr, d.Nd, second != nullptr, sizeof(R)), ctx->s>>>(
+    launch(ctx, k_rhs_par<R>, (d.P + ppb - 1) / ppb, (second ? 6 : 4) * tw, rhs_par_smem(d.Nr, d.Nd, second != nullptr, sizeof(R)),
         ctx->geom(), rp, par_tables(ctx), reinterpret_cast<const V*>(ctx->AR),
         reinterpret_cast<const double2*>(x), reinterpret_cast<const double2*>(second), u_orig, out, ppb, tw);
     CK(cudaGetLastError());
     return RSC_OK;
   }
-  k_rhs<R><<<(d.P + PPB - 1) / PPB, dim3(round32(d.Nr), PPB), smem, ctx->s>>>(
+  launch(ctx, k_rhs<R>, (d.P + PPB - 1) / PPB, dim3(round32(d.Nr), PPB), smem,
       ctx->geom(), rp, reinterpret_cast<const V*>(ctx->AR), reinterpret_cast<const double2*>(x),
       reinterpret_cast<const double2*>(U), u_orig,
       reinterpret_cast<const double2*>(xe ? xe : x), out);
@@ -1421,13 +1447,13 @@ cudaError_t launch_chain_async_q(rsc_ctx* ctx, const ChainBlocks& cb, double* ou
   cfg.blockDim = dim3(32 * NS * ((RPC + 3) / 4));
   cfg.dynamicSmemBytes = chain_smem_async(d, CS, outward, NS);
   cfg.stream = ctx->s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 1 + early_attr(ctx, attr + 1);
   const int cap = chain_steps_cap(d);
   if (outward)
     return cudaLaunchKernelEx(&cfg, k_chain_out_async<Q / NS, NS>, ctx->geom(), cb.off, cb.H, cb.W,
@@ -1452,13 +1478,13 @@ cudaError_t launch_chain_q(rsc_ctx* ctx, const ChainBlocks& cb, double* out, boo
   cfg.blockDim = dim3(32 * ((RPC + 3) / 4));
   cfg.dynamicSmemBytes = chain_smem(d, CS, outward);
   cfg.stream = ctx->s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 1 + early_attr(ctx, attr + 1);
   if (outward)
     return cudaLaunchKernelEx(&cfg, k_chain_out<Q>, ctx->geom(), cb.off, cb.H, cb.W,
                               reinterpret_cast<double2*>(out), (const double2*)ctx->mid, CS, cb.bs);
@@ -1492,13 +1518,13 @@ cudaError_t launch_chain_df_q(rsc_ctx* ctx, const DevFactor* f, double* out, boo
   cfg.blockDim = dim3(32 * NS * ((RPC + 3) / 4));
   cfg.dynamicSmemBytes = chain_smem_async(d, CS, outward, NS);
   cfg.stream = ctx->s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 1 + early_attr(ctx, attr + 1);
   const int cap = chain_steps_cap(d);
   const long* off = cr ? f->cr_red_off : f->chain_off;
   const float4* H = cr ? f->Hr : f->Hs;
@@ -1547,14 +1573,14 @@ void launch_cr_pass_df(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) 
   // four lanes per row, the rows in equal passes of at most 64
   const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));
   if (pass == 0)
-    k_cr_odd_df<CTAS><<<2 * ctx->n_cr_odd, thr, 2 * v, ctx->s>>>(
+    launch(ctx, k_cr_odd_df<CTAS>, 2 * ctx->n_cr_odd, thr, 2 * v,
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->rhs, ctx->cr_w);
   else if (pass == 1)
-    k_cr_even_df<CTAS><<<2 * ctx->n_cr_even, thr, 2 * v, ctx->s>>>(
+    launch(ctx, k_cr_even_df<CTAS>, 2 * ctx->n_cr_even, thr, 2 * v,
         ctx->geom(), even, f->cr_red_off, f->Gr, ctx->d_cr_rowf, ctx->d_cr_pairf, ctx->rhs,
         ctx->cr_w, o);
   else
-    k_cr_back_df<CTAS><<<2 * ctx->n_cr_odd, thr, 5 * v, ctx->s>>>(
+    launch(ctx, k_cr_back_df<CTAS>, 2 * ctx->n_cr_odd, thr, 5 * v,
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->d_cr_rowf, ctx->d_cr_pairf,
         ctx->rhs, o);
 }
@@ -1567,13 +1593,13 @@ void launch_cr_pass_64(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) 
   double2 *o = reinterpret_cast<double2*>(out), *w = reinterpret_cast<double2*>(ctx->cr_w);
   const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));   // as launch_cr_pass_df
   if (pass == 0)
-    k_cr_odd<<<2 * ctx->n_cr_odd, thr, 2 * v, ctx->s>>>(ctx->geom(), odd, f->cr_odd_off, f->D64,
+    launch(ctx, k_cr_odd, 2 * ctx->n_cr_odd, thr, 2 * v, ctx->geom(), odd, f->cr_odd_off, f->D64,
                                                         ctx->d_E01_64, ctx->rhs, w);
   else if (pass == 1)
-    k_cr_even<<<2 * ctx->n_cr_even, thr, v, ctx->s>>>(ctx->geom(), even, f->cr_red_off, f->G64,
+    launch(ctx, k_cr_even, 2 * ctx->n_cr_even, thr, v, ctx->geom(), even, f->cr_red_off, f->G64,
                                                       ctx->d_rowf64, ctx->d_pairf64, ctx->rhs, w, o);
   else
-    k_cr_back<<<2 * ctx->n_cr_odd, thr, 4 * v, ctx->s>>>(ctx->geom(), odd, f->cr_odd_off, f->D64,
+    launch(ctx, k_cr_back, 2 * ctx->n_cr_odd, thr, 4 * v, ctx->geom(), odd, f->cr_odd_off, f->D64,
                                                          ctx->d_E01_64, ctx->d_rowf64, ctx->d_pairf64,
                                                          ctx->rhs, o);
 }
@@ -1597,11 +1623,11 @@ void launch_gemv_df(rsc_ctx* ctx, const DevFactor* f, double* out) {
   const size_t sm = (size_t)d.Nr * sizeof(float4);
   double2* o = reinterpret_cast<double2*>(out);
   switch (chain_maxq(d.Nr)) {
-    case 2: k_block_gemv_df<2><<<2 * d.P, 256, sm, ctx->s>>>(ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
-    case 4: k_block_gemv_df<4><<<2 * d.P, 256, sm, ctx->s>>>(ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
-    case 8: k_block_gemv_df<8><<<2 * d.P, 256, sm, ctx->s>>>(ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
-    case 12: k_block_gemv_df<12><<<2 * d.P, 256, sm, ctx->s>>>(ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
-    default: k_block_gemv_df<16><<<2 * d.P, 256, sm, ctx->s>>>(ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
+    case 2: launch(ctx, k_block_gemv_df<2>, 2 * d.P, 256, sm, ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
+    case 4: launch(ctx, k_block_gemv_df<4>, 2 * d.P, 256, sm, ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
+    case 8: launch(ctx, k_block_gemv_df<8>, 2 * d.P, 256, sm, ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
+    case 12: launch(ctx, k_block_gemv_df<12>, 2 * d.P, 256, sm, ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
+    default: launch(ctx, k_block_gemv_df<16>, 2 * d.P, 256, sm, ctx->geom(), f->chain_off, f->Gs, ctx->rhs, o); break;
   }
 }
 
@@ -1662,7 +1688,7 @@ rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = 
     if (df)
       launch_gemv_df(ctx, f, out);
     else
-      k_block_gemv<<<2 * d.P, 256, (size_t)d.Nr * sizeof(double2), ctx->s>>>(
+      launch(ctx, k_block_gemv, 2 * d.P, 256, (size_t)d.Nr * sizeof(double2),
           ctx->geom(), f->chain_off, f->G, ctx->rhs, reinterpret_cast<double2*>(out));
     CK(cudaGetLastError());
   }
@@ -1700,6 +1726,7 @@ rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = 
   }
   if (fork) {
     CK(cudaStreamWaitEvent(ctx->s, ctx->ev_join, 0));
+    ctx->joined = true;
     return RSC_OK;
   }
   if (!temp) return RSC_OK;
@@ -1753,10 +1780,10 @@ rsc_status stage_solve_fp64(rsc_ctx* ctx, const DevFactor* f, double* out) {
       const FacGeom fg = fac_geom(ctx, f->dt);
       // the residual r is in place over b: the next one is r less the operator of the last correction
       const double2* xo = reinterpret_cast<const double2*>(it ? ctx->ref_tmp : out);
-      k_chain_products<<<(d.P + ppb - 1) / ppb, 4 * tw, 4 * (size_t)ppb * d.Nr * sizeof(double), ctx->s>>>(
+      launch(ctx, k_chain_products, (d.P + ppb - 1) / ppb, 4 * tw, 4 * (size_t)ppb * d.Nr * sizeof(double),
           fg, ctx->d_EcT0, ctx->d_EcT1, ctx->d_EcT2, ctx->d_EcT4, d.P, xo, ctx->res_z, ppb);
       CK(cudaGetLastError());
-      k_chain_residual<<<(int)(((long)d.P * d.Nr + 127) / 128), 128, 0, ctx->s>>>(
+      launch(ctx, k_chain_residual, (int)(((long)d.P * d.Nr + 127) / 128), 128, 0,
           fg, ctx->par64[4], ctx->d_rowf64, ctx->d_pairf64, ctx->d_pair_l, ctx->d_pair_m, d.P, ctx->res_z, xo,
           ctx->rhs);
       CK(cudaGetLastError());
@@ -1764,7 +1791,7 @@ rsc_status stage_solve_fp64(rsc_ctx* ctx, const DevFactor* f, double* out) {
     CKS(stage_solve(ctx, f, ctx->ref_tmp, false, false));
     {
       KSpan sp(ctx, RSC_K_BLAS, 24.0 * nef, 2.0 * nef);
-      k_axpby<<<nb, 256, 0, ctx->s>>>(1.0, ctx->ref_tmp, 1.0, out, nef);
+      launch(ctx, k_axpby, nb, 256, 0, 1.0, ctx->ref_tmp, 1.0, out, nef);
       CK(cudaGetLastError());
     }
   }
@@ -1982,7 +2009,7 @@ rsc_status do_step2(rsc_ctx* ctx, double* U, double dt) {
   CKS(stage_solve_path<R>(ctx, f, ctx->vtmp));
   {
     KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-    k_axpby<<<nb, 256, 0, ctx->s>>>(-1.0, U, 2.0, ctx->vtmp, n);
+    launch(ctx, k_axpby, nb, 256, 0, -1.0, U, 2.0, ctx->vtmp, n);
     CK(cudaGetLastError());
   }
   // corrector
@@ -1990,21 +2017,21 @@ rsc_status do_step2(rsc_ctx* ctx, double* U, double dt) {
   CKS(stage_products_analysis<R>(ctx, false));
   {
     KSpan sp(ctx, RSC_K_BLAS, 3.0 * nar * sizeof(V), 2.0 * nar);
-    k_average<R><<<nb, 256, 0, ctx->s>>>(reinterpret_cast<V*>(ctx->AR),
+    launch(ctx, k_average<R>, nb, 256, 0, reinterpret_cast<V*>(ctx->AR),
                                         reinterpret_cast<const V*>(ctx->AR0), nar);
     CK(cudaGetLastError());
   }
   CK(cudaMemcpyAsync(ctx->xtmp, U, n * sizeof(double), cudaMemcpyDeviceToDevice, ctx->s));
   {
     KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-    k_axpby<<<nb, 256, 0, ctx->s>>>(0.5, ctx->vtmp, 0.5, ctx->xtmp, n);
+    launch(ctx, k_axpby, nb, 256, 0, 0.5, ctx->vtmp, 0.5, ctx->xtmp, n);
     CK(cudaGetLastError());
   }
   CKS(stage_rhs<R>(ctx, rp, U, nullptr, nullptr, ctx->rhs, ctx->xtmp));
   CKS(stage_solve_path<R>(ctx, f, ctx->vtmp));
   {
     KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-    k_axpby<<<nb, 256, 0, ctx->s>>>(2.0, ctx->vtmp, -1.0, U, n);
+    launch(ctx, k_axpby, nb, 256, 0, 2.0, ctx->vtmp, -1.0, U, n);
     CK(cudaGetLastError());
   }
   return RSC_OK;
@@ -2047,7 +2074,7 @@ rsc_status do_jvp_eager(rsc_ctx* ctx, const double* U, double C, long J, const d
   launch_1d_grid(n, &nb);
   {
     KSpan sp(ctx, RSC_K_BLAS, 16.0 * n, 0.0);
-    k_copy_zero_slot<<<nb, 256, 0, ctx->s>>>(u, J, ctx->xtmp, n);
+    launch(ctx, k_copy_zero_slot, nb, 256, 0, u, J, ctx->xtmp, n);
     CK(cudaGetLastError());
   }
   CKS(stage_synth<R>(ctx, ctx->xtmp, ctx->FC));
@@ -2058,7 +2085,7 @@ rsc_status do_jvp_eager(rsc_ctx* ctx, const double* U, double C, long J, const d
   CKS(stage_solve_path<R>(ctx, f, out));
   {
     KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-    k_axpby<<<nb, 256, 0, ctx->s>>>(-1.0, ctx->xtmp, 1.0, out, n);
+    launch(ctx, k_axpby, nb, 256, 0, -1.0, ctx->xtmp, 1.0, out, n);
     CK(cudaGetLastError());
   }
   return RSC_OK;
@@ -2073,7 +2100,7 @@ rsc_status jvp_body_indirect(rsc_ctx* ctx, const double* U, double C, long J, De
   launch_1d_grid(n, &nb);
   {
     KSpan sp(ctx, RSC_K_BLAS, 16.0 * n, 0.0);
-    k_copy_zero_slot_ind<<<nb, 256, 0, ctx->s>>>(ctx->d_slots, J, ctx->xtmp, ctx->d_cslot, n);
+    launch(ctx, k_copy_zero_slot_ind, nb, 256, 0, ctx->d_slots, J, ctx->xtmp, ctx->d_cslot, n);
     CK(cudaGetLastError());
   }
   CKS(stage_synth<R>(ctx, ctx->xtmp, ctx->FC));
@@ -2084,7 +2111,7 @@ rsc_status jvp_body_indirect(rsc_ctx* ctx, const double* U, double C, long J, De
   CKS(stage_solve_path<R>(ctx, f, ctx->jvp_y));
   {
     KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-    k_finish_ind<<<nb, 256, 0, ctx->s>>>(ctx->d_slots, ctx->jvp_y, ctx->xtmp, n);
+    launch(ctx, k_finish_ind, nb, 256, 0, ctx->d_slots, ctx->jvp_y, ctx->xtmp, n);
     CK(cudaGetLastError());
   }
   return RSC_OK;
@@ -2110,7 +2137,9 @@ rsc_status do_jvp(rsc_ctx* ctx, const double* U, double C, long J, const double*
     const long before = ctx->launches;
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(ctx->s, cudaStreamCaptureModeThreadLocal));
+    ctx->capturing = true;
     const rsc_status st = jvp_body_indirect<R>(ctx, U, C, J, f, dt);
+    ctx->capturing = false;
     const cudaError_t ce = cudaStreamEndCapture(ctx->s, &graph);
     ctx->s = user;
     if (st != RSC_OK) {
@@ -2125,7 +2154,7 @@ rsc_status do_jvp(rsc_ctx* ctx, const double* U, double C, long J, const double*
     ctx->launches = before;
     ctx->jvp_key = {fp32, U, C, J, dt};
   }
-  k_set_ptrs<<<1, 1, 0, ctx->s>>>(ctx->d_slots, u, out);
+  launch(ctx, k_set_ptrs, 1, 1, 0, ctx->d_slots, u, out);
   CK(cudaGetLastError());
   CK(cudaGraphLaunch(ctx->jvp_exec, ctx->s));
   ctx->launches += ctx->jvp_nodes + 1;
@@ -2147,15 +2176,15 @@ rsc_status dots(rsc_ctx* ctx, const double* V, long ld, int nv, const double* w,
   {
     KSpan sp(ctx, RSC_K_DOTS, 8.0 * n * (nv + 1), 2.0 * n * nv);
     if (split)
-      k_dots_split<<<dim3(nchunk, (nv + 7) / 8), 256, 0, ctx->s>>>(V, ld, nv, w, n, ctx->partial);
+      launch(ctx, k_dots_split, dim3(nchunk, (nv + 7) / 8), 256, 0, V, ld, nv, w, n, ctx->partial);
     else
-      k_dots_tiled<<<nchunk, 256, 8 * (size_t)nv * sizeof(double), ctx->s>>>(V, ld, nv, w, n,
+      launch(ctx, k_dots_tiled, nchunk, 256, 8 * (size_t)nv * sizeof(double), V, ld, nv, w, n,
                                                                            ctx->partial);
     CK(cudaGetLastError());
   }
   {
     KSpan sp(ctx, RSC_K_DOTS, 8.0 * nv * nchunk, (double)nv * nchunk);
-    k_reduce_rows<<<nv, 256, 0, ctx->s>>>(ctx->partial, nchunk, dst);
+    launch(ctx, k_reduce_rows, nv, 256, 0, ctx->partial, nchunk, dst);
     CK(cudaGetLastError());
   }
   return RSC_OK;
@@ -2247,9 +2276,9 @@ rsc_status gmres(rsc_ctx* ctx, const double* U, double C, long J, const double* 
   {
     KSpan sp(ctx, RSC_K_BLAS, 16.0 * n, 1.0 * n);
     if (split)
-      k_scale_split<<<nb, 256, 0, ctx->s>>>(b, V, Vs, n, nullptr, 0, nullptr, 1.0 / beta);
+      launch(ctx, k_scale_split, nb, 256, 0, b, V, Vs, n, nullptr, 0, nullptr, 1.0 / beta);
     else
-      k_axpby<<<nb, 256, 0, ctx->s>>>(1.0 / beta, b, 0.0, V, n);
+      launch(ctx, k_axpby, nb, 256, 0, 1.0 / beta, b, 0.0, V, n);
     CK(cudaGetLastError());
   }
   // device buffer: [0] |w|^2 of the previous iteration, [1, k+2) s, [k+2, 2k+3) t
@@ -2273,16 +2302,16 @@ rsc_status gmres(rsc_ctx* ctx, const double* U, double C, long J, const double* 
       {
         KSpan sp(ctx, RSC_K_DOTS, 8.0 * n * (k + 3), 4.0 * n * (k + 1));
         if (split)
-          k_dots_pair_s<<<dim3(nchunk, (k + 1 + 15) / 16), 512, 0, ctx->s>>>(
+          launch(ctx, k_dots_pair_s, dim3(nchunk, (k + 1 + 15) / 16), 512, 0,
               Vs, ld, k + 1, w, Vs + (long)k * ld, ctx->partial);
         else
-          k_dots_pair<<<dim3(nchunk, (k + 1 + 15) / 16), 256, 0, ctx->s>>>(V, ld, k + 1, w, vk,
+          launch(ctx, k_dots_pair, dim3(nchunk, (k + 1 + 15) / 16), 256, 0, V, ld, k + 1, w, vk,
                                                                             ctx->partial);
         CK(cudaGetLastError());
       }
       {
         KSpan sp(ctx, RSC_K_DOTS, 16.0 * (k + 1) * nchunk, 2.0 * (k + 1) * nchunk);
-        k_reduce_rows<<<2 * (k + 1), 256, 0, ctx->s>>>(ctx->partial, nchunk, dbuf + 1);
+        launch(ctx, k_reduce_rows, 2 * (k + 1), 256, 0, ctx->partial, nchunk, dbuf + 1);
         CK(cudaGetLastError());
       }
     }
@@ -2343,24 +2372,24 @@ rsc_status gmres(rsc_ctx* ctx, const double* U, double C, long J, const double* 
     {
       KSpan sp(ctx, RSC_K_AXPY, 8.0 * n * (k + 3), 2.0 * n * (k + 2));
       if (split)
-        k_axpy_norm_s<<<nb, 256, (size_t)(k + 1) * sizeof(float2), ctx->s>>>(Vs, ld, k + 1, d_h,
+        launch(ctx, k_axpy_norm_s, nb, 256, (size_t)(k + 1) * sizeof(float2), Vs, ld, k + 1, d_h,
                                                                              w, n, ctx->partial);
       else
-        k_axpy_norm<<<nb, 256, 0, ctx->s>>>(V, ld, k + 1, d_h, w, n, ctx->partial);
+        launch(ctx, k_axpy_norm, nb, 256, 0, V, ld, k + 1, d_h, w, n, ctx->partial);
       CK(cudaGetLastError());
     }
     if (!split) {
       KSpan sp(ctx, RSC_K_BLAS, 8.0 * nb, 1.0 * nb);
-      k_reduce_rows<<<1, 256, 0, ctx->s>>>(ctx->partial, nb, dbuf);
+      launch(ctx, k_reduce_rows, 1, 256, 0, ctx->partial, nb, dbuf);
       CK(cudaGetLastError());
     }
     {
       KSpan sp(ctx, RSC_K_BLAS, 16.0 * n + 8.0 * nb, 1.0 * n);
       if (split)   // the norm's block shares are summed inside (|w|^2 to dbuf[0])
-        k_scale_split<<<nb, 256, 0, ctx->s>>>(w, w, Vs + (long)(k + 1) * ld, n, ctx->partial, nb,
+        launch(ctx, k_scale_split, nb, 256, 0, w, w, Vs + (long)(k + 1) * ld, n, ctx->partial, nb,
                                               dbuf, 1.0);
       else
-        k_scale_inv_sqrt<<<nb, 256, 0, ctx->s>>>(w, n, dbuf);
+        launch(ctx, k_scale_inv_sqrt, nb, 256, 0, w, n, dbuf);
       CK(cudaGetLastError());
     }
   }
@@ -2376,10 +2405,10 @@ rsc_status gmres(rsc_ctx* ctx, const double* U, double C, long J, const double* 
   {
     KSpan sp(ctx, RSC_K_AXPY, 8.0 * n * (kk + 2), 2.0 * n * kk);
     if (split)
-      k_multi_axpy_s<<<nb, 256, (size_t)std::max(kk, 1) * sizeof(float2), ctx->s>>>(Vs, ld, kk,
+      launch(ctx, k_multi_axpy_s, nb, 256, (size_t)std::max(kk, 1) * sizeof(float2), Vs, ld, kk,
                                                                                     d_h, x, n);
     else
-      k_multi_axpy2<<<nb, 256, 0, ctx->s>>>(V, ld, kk, d_h, 1.0, x, n);
+      launch(ctx, k_multi_axpy2, nb, 256, 0, V, ld, kk, d_h, 1.0, x, n);
     CK(cudaGetLastError());
   }
   CK(cudaStreamSynchronize(ctx->s));
@@ -3076,7 +3105,7 @@ rsc_status rsc_newton_rw(rsc_ctx* ctx, double* U, double* C, long J, const rsc_n
     CKS(step_any(ctx, ctx->rtmp, Cv, o->dt_newton, false));
     {
       KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-      k_axpby<<<nb, 256, 0, ctx->s>>>(-1.0, U, 1.0, ctx->rtmp, n);
+      launch(ctx, k_axpby, nb, 256, 0, -1.0, U, 1.0, ctx->rtmp, n);
       CK(cudaGetLastError());
     }
     double rn;
@@ -3111,7 +3140,7 @@ rsc_status rsc_newton_rw(rsc_ctx* ctx, double* U, double* C, long J, const rsc_n
     }
     {
       KSpan sp(ctx, RSC_K_BLAS, 24.0 * n, 2.0 * n);
-      k_axpby<<<nb, 256, 0, ctx->s>>>(-1.0, ctx->vtmp, 1.0, U, n);
+      launch(ctx, k_axpby, nb, 256, 0, -1.0, ctx->vtmp, 1.0, U, n);
       CK(cudaGetLastError());
     }
     Cv -= c;
@@ -3676,6 +3705,7 @@ rsc_status rsc_batch_apply_jacobian(rsc_batch* b, const double* const* U, const 
     for (int i = 0; i < n && st == RSC_OK; ++i) {
       rsc_ctx* c = b->ctx[i];
       if (cudaStreamWaitEvent(b->streams[i], b->fork, 0) != cudaSuccess) { st = RSC_ECUDA; break; }
+      c->capturing = true;
       const bool prof = c->prof_on;
       c->prof_on = false;
       const long before = c->launches;
@@ -3689,6 +3719,7 @@ rsc_status rsc_batch_apply_jacobian(rsc_batch* b, const double* const* U, const 
         st = fp32 ? do_jvp_eager<float>(c, U[i], C[i], Jq, u[i] + q * nn, out[i] + q * nn, f, dt)
                   : do_jvp_eager<double>(c, U[i], C[i], Jq, u[i] + q * nn, out[i] + q * nn, f, dt);
       }
+      c->capturing = false;
       nodes += c->launches - before;
       c->prof_on = prof;
       if (st == RSC_OK && (cudaEventRecord(b->join[i], b->streams[i]) != cudaSuccess ||

@@ -127,6 +127,7 @@ __global__ void k_chain_half_async(DevGeom g, const long* __restrict__ chain_off
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 ca_sh[];
   const ChainInfo ci = chain_info(g, chain_off, CS, bs);
+  grid_begin();
   const int Nr = ci.Nr;
   const CaLane c = ca_lane<QH, NS>(Nr, CS, (int)cluster.block_rank());
   double2* v = ca_sh;                       // [2][Nr]
@@ -209,6 +210,7 @@ __global__ void k_chain_out_async(DevGeom g, const long* __restrict__ chain_off,
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 ca_sh[];
   const ChainInfo ci = chain_info(g, chain_off, CS, bs);
+  grid_begin();
   const int Nr = ci.Nr;
   const CaLane c = ca_lane<QH, NS>(Nr, CS, (int)cluster.block_rank());
   double2* v = ca_sh;

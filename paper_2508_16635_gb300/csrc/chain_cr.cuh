@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(256, CTAS) k_cr_odd_df(DevGeom g, const int* _
   const CrBlock b = cr_block(g, odd_pairs);
   const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Di, Nr);
+  grid_begin();
   float4* sb = cr_sh;
   float4* su = cr_sh + Nr;
   for (int k = threadIdx.x; k < Nr; k += blockDim.x) sb[k] = cd_split(rhs[b.row0 + k]);
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(256, CTAS) k_cr_even_df(DevGeom g, const int* 
   const CrBlock b = cr_block(g, even_pairs);
   const float4* Gt = Gr + (red_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Gt, Nr);
+  grid_begin();
   float4* sb = cr_sh;
   float4* sy = cr_sh + Nr;
   const long half = 2L * g.P * Nr;
@@ -296,6 +298,7 @@ __global__ void __launch_bounds__(256, CTAS) k_cr_back_df(DevGeom g, const int* 
   const CrBlock b = cr_block(g, odd_pairs);
   const float4* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Di, Nr);
+  grid_begin();
   float4* y0 = cr_sh;
   float4* y1 = cr_sh + Nr;
   float4* e0 = cr_sh + 2 * Nr;

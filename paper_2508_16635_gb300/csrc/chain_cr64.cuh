@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(256, 5) k_cr_odd(DevGeom g, const int* __restr
   const CrBlock b = cr_block(g, odd_pairs);
   const double2* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Di, Nr);
+  grid_begin();
   double2* sb = cr64_sh;
   double2* su = cr64_sh + Nr;
   for (int k = threadIdx.x; k < Nr; k += blockDim.x) sb[k] = rhs[b.row0 + k];
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(256, 5) k_cr_even(DevGeom g, const int* __rest
   const CrBlock b = cr_block(g, even_pairs);
   const double2* Gt = Gr + (red_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Gt, Nr);
+  grid_begin();
   double2* sb = cr64_sh;
   const long half = 2L * g.P * Nr;
   const bool left = b.i >= 1, right = b.i + 1 <= b.nb - 1;
@@ -196,6 +198,7 @@ __global__ void __launch_bounds__(256, 5) k_cr_back(DevGeom g, const int* __rest
   const CrBlock b = cr_block(g, odd_pairs);
   const double2* Di = Dinv + (odd_off[b.c] + (b.i >> 1)) * (long)Nr * Nr;
   cr_prefetch(Di, Nr);
+  grid_begin();
   double2* y0 = cr64_sh;
   double2* y1 = cr64_sh + Nr;
   double2* e0 = cr64_sh + 2 * Nr;

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(256) k_block_gemv_df(DevGeom g, const long* __
                                                        const float4* __restrict__ G,
                                                        const double2* __restrict__ rhs,
                                                        double2* __restrict__ out) {
+  grid_begin();
   extern __shared__ float4 svf[];
   const int Nr = g.Nr, P = g.P;
   const int p = blockIdx.x >> 1, fld = blockIdx.x & 1;
@@ -218,19 +219,19 @@ __global__ void k_chain_half_df(DevGeom g, const long* __restrict__ chain_off,
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int k = threadIdx.x; k < Nr; k += blockDim.x)
-    v[k] = has ? cd_split(out[ci.row(first) + k]) : make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr int PD = CdDepth<QH>::PD;
   float4 mc[QH], mb[PD][QH];   // mb[q]: rows of block t + q (t the next step)
   double2 gb[PD];
 #pragma unroll
-  for (int q = 0; q < PD; ++q) {
-    gb[q] = make_double2(0, 0);
-    if (q + 1 <= count) {
+  for (int q = 0; q < PD; ++q)
+    if (q + 1 <= count)
       cd_load<QH>(H + (ci.boff + first + (q + 1) * step) * ci.blk, c.r, c.s, c.q0, Nr, c.active, mb[q]);
-      if (c.active) gb[q] = out[ci.row(first + (q + 1) * step) + c.r];
-    }
-  }
+  grid_begin();
+  for (int k = threadIdx.x; k < Nr; k += blockDim.x)
+    v[k] = has ? cd_split(out[ci.row(first) + k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < PD; ++q)
+    gb[q] = q + 1 <= count && c.active ? out[ci.row(first + (q + 1) * step) + c.r] : make_double2(0, 0);
   cluster.sync();   // barriers initialised and v[0] loaded everywhere before any st.async
   bool ok = true;
   for (int t = 1; t <= count; ++t) {
@@ -312,6 +313,7 @@ __global__ void k_chain_out_df(DevGeom g, const long* __restrict__ chain_off,
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  grid_begin();
   for (int k = threadIdx.x; k < Nr; k += blockDim.x) {
     yup[k] = cd_split(mc0[k]);
     zdn[k] = cd_split(mc0[Nr + k]);

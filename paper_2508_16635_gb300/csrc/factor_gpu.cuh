@@ -486,6 +486,7 @@ __global__ void __launch_bounds__(640) k_chain_products(FacGeom g, const double*
                                                         const double* __restrict__ E4T, int P,
                                                         const double2* __restrict__ x, double2* __restrict__ Z,
                                                         int PPB) {
+  grid_begin();
   extern __shared__ double cp_sh[];   // [group][pl][k]
   const int Nr = g.Nr, NH = (Nr + 1) / 2;
   const int pb = blockIdx.x * PPB, np = min(PPB, P - pb);
@@ -531,6 +532,7 @@ __global__ void k_chain_residual(FacGeom g, const double* __restrict__ irc, cons
                                  const CrPair* __restrict__ pairf, const int* __restrict__ pair_l,
                                  const int* __restrict__ pair_m, int P, const double2* __restrict__ Z,
                                  const double2* __restrict__ x, double2* __restrict__ rb) {
+  grid_begin();
   const int Nr = g.Nr;
   const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long)P * Nr) return;

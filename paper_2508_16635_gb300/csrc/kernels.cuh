@@ -20,6 +20,20 @@
 
 namespace rsc {
 
+// Start of a kernel that may be launched while the kernel ahead of it in its stream ends (launch() in
+// capi.cu): waits until that one has ended and its results are visible.  Nothing that a kernel of the
+// stream writes is touched before this; the factors and index tables of the chain solve, complete
+// since their factorisation, may be (their blocks are on the way to L2 by then).
+// A step is a chain of dependent kernels, 5 to 40 us each at L = 127, and between the last CTA of
+// one and the first load of the next the device did nothing.  Measured (one GB300): steps at
+// L = 7 76 -> 57 us, ten monitored FP64 steps at L = 31 2438 -> 2033, four second-order steps at L = 52
+// 1270 -> 1094, ten mixed steps at L = 127 2650 -> 2462, two FP64 2003 -> 1947, L = 255 7863 -> 7785 us.
+// A kernel does not release the next one early: its CTAs then took the free slots of whichever SMs
+// had any, and one-wave kernels ran unevenly (L = 127 mixed 2730, FP64 2226 us).
+__device__ __forceinline__ void grid_begin() {
+  cudaGridDependencySynchronize();
+}
+
 template <typename R> struct C2;
 template <> struct C2<double> { using T = double2; };
 template <> struct C2<float> { using T = float2; };
@@ -98,6 +112,7 @@ template <> struct Tab<float> {
 template <typename R>
 __global__ void k_radial(DevGeom g, const double2* __restrict__ x,
                          typename C2<R>::T* __restrict__ SR) {
+  grid_begin();
   using V = typename C2<R>::T;
   extern __shared__ unsigned char sh_raw[];
   V* sc = reinterpret_cast<V*>(sh_raw);  // [3][Nr] coefficients in precision R
@@ -149,6 +164,7 @@ __global__ void k_radial(DevGeom g, const double2* __restrict__ x,
 template <typename R>
 __global__ void k_analysis(DevGeom g, DevLegendre<R> T, const typename C2<R>::T* __restrict__ FA,
                            typename C2<R>::T* __restrict__ AR, int TC) {
+  grid_begin();
   using V = typename C2<R>::T;
   extern __shared__ unsigned char sh_raw[];
   const int n2 = g.nlat2, nlat = g.nlat, K1 = g.K + 1, Nd = g.Nd;
@@ -245,6 +261,7 @@ __global__ void k_rhs(DevGeom g, RhsParams rp, const typename C2<R>::T* __restri
                       const double2* __restrict__ x, const double2* __restrict__ U,
                       const double* __restrict__ u_orig, const double2* __restrict__ xe,
                       double2* __restrict__ rhs) {
+  grid_begin();
   const int has_c = rp.J >= 0;
   using V = typename C2<R>::T;
   extern __shared__ double2 sh2[];
@@ -507,6 +524,7 @@ __global__ void k_rhs(DevGeom g, RhsParams rp, const typename C2<R>::T* __restri
 template <typename R>
 __global__ void k_average(typename C2<R>::T* __restrict__ a, const typename C2<R>::T* __restrict__ b,
                           long n) {
+  grid_begin();
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     typename C2<R>::T v = a[i];
     const typename C2<R>::T w = b[i];
@@ -540,6 +558,7 @@ __device__ __forceinline__ double2 cmac(double2 acc, double2 a, double2 b) {
 __global__ void k_block_gemv(DevGeom g, const long* __restrict__ chain_off,
                              const double2* __restrict__ G, const double2* __restrict__ rhs,
                              double2* __restrict__ out) {
+  grid_begin();
   extern __shared__ double2 sv[];
   const int Nr = g.Nr, P = g.P;
   const int p = blockIdx.x >> 1, fld = blockIdx.x & 1;
@@ -674,6 +693,7 @@ template <int MAXQ>
 __global__ void k_chain_half(DevGeom g, const long* __restrict__ chain_off,
                              const double2* __restrict__ H, double2* __restrict__ out,
                              double2* __restrict__ mid, int CS, int bs) {
+  grid_begin();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 sv[];  // [2][Nr] ping-pong, then hist[steps][RPC]
@@ -741,6 +761,7 @@ template <int MAXQ>
 __global__ void k_chain_out(DevGeom g, const long* __restrict__ chain_off,
                             const double2* __restrict__ H, const double2* __restrict__ W,
                             double2* __restrict__ out, const double2* __restrict__ mid, int CS, int bs) {
+  grid_begin();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ double2 sv[];  // [2][Nr] ping-pong, [2][Nr] middle inputs, hist[steps][RPC]
@@ -846,6 +867,7 @@ __global__ void k_temp_solve(DevGeom g, const double* __restrict__ Tinv,
 __global__ void __launch_bounds__(256) k_dots_tiled(const double* __restrict__ V, long ld, int nv,
                                                     const double* __restrict__ w, long n,
                                                     double* __restrict__ partial) {
+  grid_begin();
   extern __shared__ double red2[];   // [8 warps][nv]
   const long base = (long)blockIdx.x * 2048;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -902,6 +924,7 @@ __global__ void __launch_bounds__(256) k_dots_tiled(const double* __restrict__ V
 __global__ void __launch_bounds__(256) k_dots_split(const double* __restrict__ V, long ld, int nv,
                                                     const double* __restrict__ w, long n,
                                                     double* __restrict__ partial) {
+  grid_begin();
   __shared__ double red[8][8];
   const long base = (long)blockIdx.x * 4096;
   const int j0 = blockIdx.y * 8;
@@ -963,6 +986,7 @@ __global__ void __launch_bounds__(256) k_dots_pair(const double* __restrict__ V,
                                                    const double* __restrict__ w,
                                                    const double* __restrict__ q,
                                                    double* __restrict__ partial) {
+  grid_begin();
   constexpr int E2 = 512, PER = E2 / 32;
   __shared__ double2 ws[E2], qs[E2];
   const long b2 = (long)blockIdx.x * E2;
@@ -1009,6 +1033,7 @@ __global__ void __launch_bounds__(256) k_axpy_norm(const double* __restrict__ V,
                                                    const double* __restrict__ h,
                                                    double* __restrict__ w, long n,
                                                    double* __restrict__ partial) {
+  grid_begin();
   __shared__ double red[8];
   const long n2 = n >> 1;
   double2* w2 = reinterpret_cast<double2*>(w);
@@ -1052,6 +1077,7 @@ __global__ void __launch_bounds__(256) k_axpy_norm(const double* __restrict__ V,
 
 // w <- w / sqrt(nrm2[0]) (left unchanged when nrm2[0] is zero: a breakdown the host sees).
 __global__ void k_scale_inv_sqrt(double* __restrict__ w, long n, const double* __restrict__ nrm2) {
+  grid_begin();
   // one FP64 square root and division per block (the FP64 pipe is narrow)
   __shared__ double sinv;
   const double s2 = nrm2[0];
@@ -1069,6 +1095,7 @@ __global__ void k_scale_inv_sqrt(double* __restrict__ w, long n, const double* _
 __global__ void k_multi_axpy2(const double* __restrict__ V, long ld, int nv,
                               const double* __restrict__ coef, double sign, double* __restrict__ w,
                               long n) {
+  grid_begin();
   const long n2 = n >> 1;
   double2* w2 = reinterpret_cast<double2*>(w);
   for (long i2 = (long)blockIdx.x * blockDim.x + threadIdx.x; i2 < n2;
@@ -1100,6 +1127,7 @@ __global__ void k_multi_axpy2(const double* __restrict__ V, long ld, int nv,
 
 // out[j] = sum_b partial[j * nblk + b].  grid = nv, block = 256.
 __global__ void k_reduce_rows(const double* __restrict__ partial, int nblk, double* __restrict__ out) {
+  grid_begin();
   __shared__ double red[32];
   const int j = blockIdx.x;
   double s = 0.0;
@@ -1119,6 +1147,7 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int nblk, doub
 // y = a * x + b * y
 __global__ void k_axpby(double a, const double* __restrict__ x, double b, double* __restrict__ y,
                         long n) {
+  grid_begin();
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
        idx += (long)gridDim.x * blockDim.x)
     y[idx] = a * x[idx] + b * y[idx];
@@ -1127,6 +1156,7 @@ __global__ void k_axpby(double a, const double* __restrict__ x, double b, double
 // Graph-replayed Jacobian action: the input and output vectors are reached
 // through pointers held in device memory (set by k_set_ptrs before each replay).
 __global__ void k_set_ptrs(const double** slots, const double* u, double* out) {
+  grid_begin();
   slots[0] = u;
   slots[1] = out;
 }
@@ -1134,6 +1164,7 @@ __global__ void k_set_ptrs(const double** slots, const double* u, double* out) {
 // x = u with u_J zeroed; c = u_J stored in cslot[0] (Sec. 3.4)
 __global__ void k_copy_zero_slot_ind(const double* const* slots, long J, double* __restrict__ x,
                                      double* __restrict__ cslot, long n) {
+  grid_begin();
   const double* u = slots[0];
   if (J >= 0 && blockIdx.x == 0 && threadIdx.x == 0) cslot[0] = u[J];
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
@@ -1144,6 +1175,7 @@ __global__ void k_copy_zero_slot_ind(const double* const* slots, long J, double*
 // out = y - x through the output pointer slot
 __global__ void k_finish_ind(const double* const* slots, const double* __restrict__ y,
                              const double* __restrict__ x, long n) {
+  grid_begin();
   double* out = const_cast<double*>(slots[1]);
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
        idx += (long)gridDim.x * blockDim.x)
@@ -1153,6 +1185,7 @@ __global__ void k_finish_ind(const double* const* slots, const double* __restric
 // copy with u_J zeroed (x holds the canonical layout)
 __global__ void k_copy_zero_slot(const double* __restrict__ u, long J, double* __restrict__ x,
                                  long n) {
+  grid_begin();
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
        idx += (long)gridDim.x * blockDim.x)
     x[idx] = (idx == J) ? 0.0 : u[idx];

@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(256) k_scale_split(const double* in, double* o
                                                      float2* __restrict__ outs, long n,
                                                      const double* __restrict__ part, int np,
                                                      double* __restrict__ nrm2_out, double s) {
+  grid_begin();
   if (part) {
     __shared__ double red[8];
     __shared__ double sc;
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(512) k_dots_pair_s(const float2* __restrict__ 
                                                      int nv, const double* __restrict__ w,
                                                      const float2* __restrict__ qs,
                                                      double* __restrict__ partial) {
+  grid_begin();
   constexpr int E2 = 512, PER = E2 / 32;
   __shared__ float4 ws[E2], qsh[E2];
   const long b2 = (long)blockIdx.x * E2;
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(256) k_axpy_norm_s(const float2* __restrict__ 
                                                      int nv, const double* __restrict__ h,
                                                      double* __restrict__ w, long n,
                                                      double* __restrict__ partial) {
+  grid_begin();
   extern __shared__ float2 hs[];
   __shared__ double red[8];
   for (int j = threadIdx.x; j < nv; j += blockDim.x) {
@@ -194,6 +197,7 @@ __global__ void __launch_bounds__(256) k_axpy_norm_s(const float2* __restrict__ 
 __global__ void __launch_bounds__(256) k_multi_axpy_s(const float2* __restrict__ Vs, long ld,
                                                       int nv, const double* __restrict__ coef,
                                                       double* __restrict__ x, long n) {
+  grid_begin();
   extern __shared__ float2 cs[];
   for (int j = threadIdx.x; j < nv; j += blockDim.x) {
     float a, b;

@@ -201,6 +201,7 @@ __host__ __device__ constexpr size_t tc_synth_smem(int kmax, bool pipe) {
 template <bool PIPE>
 __global__ void __launch_bounds__(kTcThreads) k_synth_tc(DevGeom g, TcTables tt, const float2* __restrict__ SR,
                                                   float2* __restrict__ FC) {
+  grid_begin();
   extern __shared__ __align__(1024) unsigned char tc_raw[];
   const int a = blockIdx.x;
   const int i0 = blockIdx.y * kTcRadii;

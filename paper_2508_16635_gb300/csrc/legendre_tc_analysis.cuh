@@ -58,6 +58,7 @@ inline size_t ta_smem() {
 __global__ void __launch_bounds__(kTaThreads) k_analysis_tc(DevGeom g, TaTables tt,
                                                      const float2* __restrict__ FA,
                                                      float2* __restrict__ AR) {
+  grid_begin();
   extern __shared__ __align__(1024) unsigned char ta_raw[];
   const int a = blockIdx.x;
   const int i0 = blockIdx.y * kTaRadii;

@@ -109,6 +109,7 @@ template <typename R, int MODE, bool EVEN, int J>
 __global__ void __launch_bounds__(prod_max_threads<R>(), 2)
 k_products(DevGeom g, DevLegendre<R> T, R Ek, const typename C2<R>::T* __restrict__ FC,
            typename C2<R>::T* __restrict__ FA, R* __restrict__ UG, int LT, int S, int Q) {
+  grid_begin();
   using V = typename C2<R>::T;
   constexpr int NK = EVEN ? 4 : 2, NPT = EVEN ? 4 : 2;
   extern __shared__ __align__(16) unsigned char pr_sh[];

@@ -72,6 +72,7 @@ __host__ __forceinline__ size_t rhs_lin_smem(int Nr, int Nd) {
 template <int NR_, int ND_>
 __global__ void __launch_bounds__(1024) k_radial_f32(DevGeom g, const double2* __restrict__ x,
                                                      float2* __restrict__ SR) {
+  grid_begin();
   extern __shared__ __align__(16) float rr_sh[];
   constexpr bool FIX = NR_ > 0;
   static_assert(!FIX || (NR_ % 4 == 0 && ND_ % 4 == 0), "fixed sizes are multiples of 4");
@@ -154,6 +155,7 @@ __global__ void __launch_bounds__(512) k_rhs_lin(DevGeom g, RhsParams rp,
                                                   const double2* __restrict__ U,
                                                   const double* __restrict__ u_orig,
                                                   double2* __restrict__ rhs) {
+  grid_begin();
   extern __shared__ __align__(16) float rl_sh[];
   constexpr bool FIX = NR_ > 0;
   static_assert(!FIX || (NR_ % 4 == 0 && ND_ % 4 == 0), "fixed sizes are multiples of 4");

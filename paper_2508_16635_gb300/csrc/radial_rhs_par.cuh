@@ -82,6 +82,7 @@ __device__ __forceinline__ void par_rows(double* z, int n, int j, double se, dou
 // half sum real parts, of the second imaginary ones; thread l of a half = (pair l / NdH, row l % NdH).
 __global__ void __launch_bounds__(320) k_radial_par(DevGeom g, ParTables pt, const double2* __restrict__ x,
                                                     double2* __restrict__ SR, int PPB) {
+  grid_begin();
   extern __shared__ double pa_sh[];
   const int Nr = g.Nr, Nd = g.Nd, P = g.P, NH = (Nd + 1) / 2;
   double* xs = pa_sh;                       // [part][pl][f][k]
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(960) k_rhs_par(DevGeom g, RhsParams rp, ParTab
                                                  const double2* __restrict__ x, const double2* __restrict__ U2,
                                                  const double* __restrict__ u_orig, double2* __restrict__ rhs,
                                                  int PPB, int TW) {
+  grid_begin();
   using V = typename C2<R>::T;
   extern __shared__ double pa_sh[];
   const int Nr = g.Nr, Nd = g.Nd, P = g.P, NH = (Nr + 1) / 2, DH = (Nd + 1) / 2;

@@ -359,6 +359,7 @@ __device__ __forceinline__ int ss_comp(bool vec, int c) {
 __global__ void __launch_bounds__(kSsThreads, 1) k_synth_sl(DevGeom g, SlTables tt, int nst,
                                                          const double2* __restrict__ SR,
                                                          double2* __restrict__ FC) {
+  grid_begin();
   extern __shared__ __align__(1024) unsigned char sl_raw[];
   const int a = blockIdx.y, i0 = blockIdx.x * kSsRad, mt = blockIdx.z;
   const int m = g.m_of[a], p0 = g.pstart[a], nl = g.L - m + 1, Nd = g.Nd;
@@ -621,6 +622,7 @@ __host__ __device__ constexpr size_t sa_smem(int ks, int nst) {
 __global__ void __launch_bounds__(kSaThreads, 1) k_analysis_sl(DevGeom g, SlTables tt, int nst,
                                                             const double2* __restrict__ FA,
                                                             double2* __restrict__ AR) {
+  grid_begin();
   extern __shared__ __align__(1024) unsigned char sl_raw[];
   const int a = blockIdx.y, i0 = blockIdx.x * kSaRad;
   const int m = g.m_of[a], p0 = g.pstart[a], nl = g.L - m + 1, Nd = g.Nd;

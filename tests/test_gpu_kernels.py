@@ -146,3 +146,24 @@ def test_chain_residual(torch, L, Ms, Nr):
         assert fwd < 1e-11
         assert fwd_T < 1e-12
     gpu.close()
+
+
+# Kernels that start while the one ahead ends: steps in a row, with nothing between the launches, give the
+# bits of traced ones (an event before and after every launch, the temperature solve in line).
+@pytest.mark.parametrize("L,Ms,Nr,n", [(7, 4, 10, 40), (31, 4, 24, 10), (52, 8, 60, 4)])
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_launches_in_a_row_and_one_by_one(torch, L, Ms, Nr, n, precision):
+    from paper_2508_16635_gb300 import RotatingShell
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0, precision=precision)
+    U0 = gpu.conductive_state() + torch.tensor(si.perturbation(L, Ms, Nr, seed=47, amp=3e-2), device="cuda")
+    out = []
+    for traced in (False, True):
+        U = U0.clone()
+        gpu.profile(traced)
+        for _ in range(n):
+            gpu.step(U, 1e-3)
+        torch.cuda.synchronize()
+        gpu.profile(False)
+        out.append(U)
+    assert torch.equal(out[0], out[1])
+    gpu.close()
