@@ -191,7 +191,8 @@ rsc_status rsc_implicit_solve(rsc_ctx* ctx, const double* rhs, double* x, double
 rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, double* out_host);
 
 /* Wall time (s) of the context's last factorisation and whether it ran on the GPU: the temperature
- * operators and, where a solve needs them, the unreduced chains.                           */
+ * operators, the unreduced chains if they were built, and on FP64 contexts the reduced chains
+ * (mixed contexts: rsc_factor_time_cr).                                                     */
 rsc_status rsc_factor_time(const rsc_ctx* ctx, double* seconds, int* on_gpu);
 /* The same for the context's last factorisation of the odd-even reduced chains
  * (rsc_tuning chain_cr; 0 s until one has run).                                  */

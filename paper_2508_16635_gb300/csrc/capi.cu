@@ -1143,8 +1143,10 @@ rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
   std::unique_lock<std::mutex> lock;
   if (ctx->share) lock = std::unique_lock<std::mutex>(ctx->share->mu);
   if (f->G) return RSC_OK;
+  const auto t0 = std::chrono::steady_clock::now();
   const rsc_status st = gpu_factor(ctx, f->dt, *f);
   if (st != RSC_OK) free_unreduced(*f);
+  ctx->factor_s += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   return st;
 }
 
@@ -3214,7 +3216,7 @@ rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, doub
 
 rsc_status rsc_factor_time(const rsc_ctx* ctx, double* seconds, int* on_gpu) {
   if (!ctx) return RSC_EINVAL;
-  if (seconds) *seconds = ctx->factor_s;
+  if (seconds) *seconds = ctx->factor_s + (ctx->p.precision == RSC_MIXED ? 0.0 : ctx->factor_cr_s);
   if (on_gpu) *on_gpu = ctx->factor_on_gpu;
   return RSC_OK;
 }
