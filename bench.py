@@ -272,7 +272,7 @@ NCU_TRAFFIC_MB = {
     # the sweeps over the odd-even reduced chains: k_chain_half_df<2, 4>: 45.5 + 0.0 MB,
     # k_chain_out_df<2, 4>: 51.3 + 18.7 MB
     ("chain_sweep", "df_cr"): 57.7,
-    # k_cr_odd_df<8>: 49.9 + 1.3 MB, k_cr_even_df<8>: 51.4 + 2.0 MB, k_cr_back_df<8>: 50.7 + 1.0 MB
+    # k_cr_odd_df: 49.9 + 1.3 MB, k_cr_even_df: 51.4 + 2.0 MB, k_cr_back_df: 50.7 + 1.0 MB
     ("chain_reduced", "df_cr"): 52.1,
 }
 
@@ -280,7 +280,8 @@ NCU_TRAFFIC_MB = {
 def traffic_variant(name, precision, tuning, dfk):
     """The NCU_TRAFFIC_MB variant of a kernel class under this tuning."""
     if name not in dfk:
-        return "fp64"
+        # FP64 solves run on reduced chains where the chains are whole (no capture of those sweeps)
+        return "fp64_cr" if name == "chain_sweep" and tuning.get("chain_parts") == 1 else "fp64"
     if precision == "mixed" and tuning.get("chain_cr", 0) and name in ("chain_sweep", "chain_reduced"):
         return "df_cr"
     return "df"
