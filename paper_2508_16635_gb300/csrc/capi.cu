@@ -23,7 +23,6 @@
 #include "chain_async.cuh"
 #include "legendre_tc.cuh"
 #include "legendre_tc_analysis.cuh"
-#include "slices_tc.cuh"
 #include "krylov_split.cuh"
 #include "chain_df.cuh"
 #include "chain_cr.cuh"
@@ -168,9 +167,7 @@ struct rsc_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool joined = false;      // the next launch follows work of the second stream
   bool capturing = false;   // the stream is captured into a graph
-  // radii per block of the CUDA-core FP32 analysis ([1]); the FP64 transforms have one shape and
-  // carry their rsc_tuning fields only
-  int rt_synth[2] = {1, 1}, rt_anal[2] = {1, 1};
+  int rt_synth[2] = {1, 1}, rt_anal[2] = {1, 1};  // radii per block, [fp64, fp32]
   int radial_f32_grid = 0, rhs_lin_grid = 0;     // persistent FP32 radial kernels (0: not used)
   int wpb[2] = {0, 0};     // warps per block of the products kernel (0: largest that fits)
   int ppb[2] = {0, 0};     // pairs per block of the right-hand-side kernel (0: 256 / Nr)
@@ -188,8 +185,6 @@ struct rsc_ctx {
   int tc_nmt = 1;
   int tc_kmax = 0;          // largest padded K of the synthesis tiles
   int synth_pipe = 0;       // 1: two-stage tensor-core synthesis (where it fits)
-  // FP64 synthesis [0] and analysis [1] on digit slices (slices_tc.cuh): tables, ring stages
-  struct { unsigned char* tiles = nullptr; long* off = nullptr; int* ea = nullptr; int nt = 1, ks = 0, nst = 0; } sl[2];
   int* d_status = nullptr;
   // tracing: launch counter, per-kernel CUDA-event timing and algorithmic traffic
   long launches = 0;
@@ -593,49 +588,6 @@ ParTables par_tables(const rsc_ctx* ctx) {
                    ctx->par32[2], ctx->par32[3], ctx->par64[4], ctx->par64[5], ctx->p.Ra / ctx->d.r_out};
 }
 
-// Digit tables of the FP64 Legendre transforms (slices_tc.cuh), cut on the device from the FP64
-// tables, which nothing else reads and which are released.
-template <bool ANAL>
-rsc_status build_slice_tables(rsc_ctx* ctx) {
-  const Dims& d = ctx->d;
-  auto& sl = ctx->sl[ANAL ? 1 : 0];
-  sl.nt = ANAL ? 1 : (d.nlat2 + 127) / 128;
-  std::vector<long> off((size_t)d.nm * 6 * sl.nt);
-  long total = 0;
-  sl.ks = 0;
-  for (int a = 0; a < d.nm; ++a)
-    for (int s = 0; s < 2; ++s) {
-      const int deg = (d.L - ctx->t.m_of[a] + 1 - s + 1) / 2;
-      const int nrow = ANAL ? deg : d.nlat2, ks = ((ANAL ? d.nlat2 : deg) + 15) / 16;
-      sl.ks = std::max(sl.ks, ks);
-      for (int w = 0; w < 3; ++w)
-        for (int t = 0; t < sl.nt; ++t) {
-          off[((size_t)(a * 2 + s) * 3 + w) * sl.nt + t] = total;
-          const int rows = std::min(128, std::max(0, nrow - 128 * t));
-          total += (long)ks * kSl * ((rows + 7) / 8) * 256;
-        }
-    }
-  CKS(upload(ctx, &sl.off, off.data(), off.size()));
-  CK(cudaMalloc(&sl.tiles, std::max<long>(total, 1)));
-  const size_t nea = (size_t)d.nm * 3 * (ANAL ? d.L + 1 : d.nlat2);
-  CK(cudaMalloc(&sl.ea, nea * sizeof(int)));
-  const SlTables tt{sl.tiles, sl.off, sl.ea, sl.nt, sl.ks, nullptr};
-  double* const* T = ctx->leg64.buf + (ANAL ? 3 : 0);
-  k_slice_exponents<ANAL><<<dim3(d.nm, 3), 256, 0, ctx->s>>>(ctx->geom(), T[0], T[1], T[2], sl.ea);
-  k_slice_tables<ANAL><<<dim3(d.nm * 6, sl.nt), 256, 0, ctx->s>>>(ctx->geom(), T[0], T[1], T[2], tt, sl.tiles);
-  CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(ctx->s));
-  for (int q = 0; q < 3; ++q) {
-    cudaFree(T[q]);
-    ctx->leg64.buf[(ANAL ? 3 : 0) + q] = nullptr;
-  }
-  // ring stages beside the resident data digits
-  const size_t lim = 227 * 1024;
-  for (sl.nst = 4; sl.nst > 2 && (ANAL ? sa_smem(sl.ks, sl.nst) : ss_smem(sl.ks, sl.nst)) > lim; --sl.nst) {
-  }
-  return RSC_OK;
-}
-
 // Whether `threads` threads of `fn` fit the register file and the block size limit.
 bool threads_fit(const void* fn, int threads) {
   cudaFuncAttributes at{};
@@ -726,6 +678,9 @@ rsc_status set_smem_limits(rsc_ctx* ctx) {
       --rt;
     return rt;
   };
+  ctx->rt_synth[0] = rt_for((const void*)k_synth<double>, round32(ctx->d.nlat2));
+  ctx->rt_synth[1] = rt_for((const void*)k_synth<float>, round32(ctx->d.nlat2));
+  ctx->rt_anal[0] = rt_for((const void*)k_analysis<double>, round32(ctx->d.L + 1));
   ctx->rt_anal[1] = rt_for((const void*)k_analysis<float>, round32(ctx->d.L + 1));
   // pairs per block of the right-hand side: 256 / Nr, halved until the registers fit
   for (int p = 0; p < 2; ++p) {
@@ -734,8 +689,9 @@ rsc_status set_smem_limits(rsc_ctx* ctx) {
     while (q > 1 && !threads_fit(fn, round32(ctx->d.Nr) * q)) q /= 2;
     ctx->ppb[p] = q;
   }
-  CK(cudaFuncSetAttribute(k_synth_sl, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  CK(cudaFuncSetAttribute(k_analysis_sl, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CK(cudaFuncSetAttribute(k_synth<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  CK(cudaFuncSetAttribute(k_synth<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  CK(cudaFuncSetAttribute(k_analysis<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   CK(cudaFuncSetAttribute(k_analysis<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   CK(cudaFuncSetAttribute(k_rhs<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   CK(cudaFuncSetAttribute(k_rhs<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
@@ -1258,10 +1214,10 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
                                                      reinterpret_cast<float2*>(FCout));
     CK(cudaGetLastError());
   } else {
-    const auto& sl = ctx->sl[0];
-    const SlTables tt{sl.tiles, sl.off, sl.ea, sl.nt, sl.ks, ctx->d_status};
-    launch(ctx, k_synth_sl, dim3((d.Nd + kSsRad - 1) / kSsRad, d.nm, sl.nt), kSsThreads, ss_smem(sl.ks, sl.nst),
-        g, tt, sl.nst, reinterpret_cast<const double2*>(ctx->SR), reinterpret_cast<double2*>(FCout));
+    const int RT = ctx->rt_synth[0];
+    launch(ctx, k_synth<R>, dim3(d.nm, (d.Nd + RT - 1) / RT), dim3(round32(d.nlat2), RT),
+        (size_t)RT * (d.L + 1) * 8 * sizeof(V) + 16 * 3 * (size_t)d.nlat2 * sizeof(R),
+        g, L.view(), reinterpret_cast<const V*>(ctx->SR), reinterpret_cast<V*>(FCout));
     CK(cudaGetLastError());
   }
   }
@@ -1343,20 +1299,16 @@ rsc_status stage_products_analysis(rsc_ctx* ctx, bool lin) {
            4.0 * d.Nd * K1 * d.nlat * sizeof(V) + 4.0 * d.P * d.Nd * sizeof(V) +
                3.0 * d.P * d.nlat2 * sizeof(R),
            24.0 * d.P * d.nlat2 * d.Nd);
-  if constexpr (sizeof(R) == 8) {
-    const auto& sl = ctx->sl[1];
-    const SlTables ta{sl.tiles, sl.off, sl.ea, sl.nt, sl.ks, ctx->d_status};
-    launch(ctx, k_analysis_sl, dim3((d.Nd + kSaRad - 1) / kSaRad, d.nm), kSaThreads, sa_smem(sl.ks, sl.nst),
-        g, ta, sl.nst, reinterpret_cast<const double2*>(ctx->FA), reinterpret_cast<double2*>(ctx->AR));
-  } else if (ctx->anal_tc) {
+  const int RTa = ctx->rt_anal[sizeof(R) == 4 ? 1 : 0];
+  const int TC = ctx->atc[sizeof(R) == 4 ? 1 : 0];
+  if (sizeof(R) == 4 && ctx->anal_tc) {
     TaTables ta{ctx->ta_tiles, ctx->ta_off, ctx->ta_nchunk, ctx->d_status};
     launch(ctx, k_analysis_tc, dim3(d.nm, (d.Nd + kTaRadii - 1) / kTaRadii), kTaThreads, ta_smem(),
         g, ta, reinterpret_cast<const float2*>(ctx->FA), reinterpret_cast<float2*>(ctx->AR));
   } else {
-    const int RTa = ctx->rt_anal[1], TC = ctx->atc[1];
-    launch(ctx, k_analysis<float>, dim3(d.nm, (d.Nd + RTa - 1) / RTa), dim3(round32(d.L + 1), RTa), analysis_smem<float>(d, RTa, TC),
-        g, leg<float>(ctx).view(), reinterpret_cast<const float2*>(ctx->FA),
-        reinterpret_cast<float2*>(ctx->AR), TC);
+    launch(ctx, k_analysis<R>, dim3(d.nm, (d.Nd + RTa - 1) / RTa), dim3(round32(d.L + 1), RTa),
+        analysis_smem<R>(d, RTa, TC), g, L.view(), reinterpret_cast<const V*>(ctx->FA),
+        reinterpret_cast<V*>(ctx->AR), TC);
   }
   CK(cudaGetLastError());
   }
@@ -2440,7 +2392,8 @@ bool tuning_ok(rsc_ctx* ctx, const rsc_tuning& t) {
     const size_t sm = p ? products_smem<float>(d, true, t.products_warps[p])
                         : products_smem<double>(d, true, t.products_warps[p]);
     if (sm > 190 * 1024) return false;
-    const int ra = p ? radii_limit((const void*)k_analysis<float>, round32(d.L + 1)) : 4;
+    const int ra = radii_limit(p ? (const void*)k_analysis<float> : (const void*)k_analysis<double>,
+                               round32(d.L + 1));
     if (t.analysis_radii[p] < 1 || t.analysis_radii[p] > ra) return false;
     if (t.analysis_chunk[p] < 1) return false;
     if (!pow2(t.products_lats[p], 16)) return false;
@@ -2454,7 +2407,8 @@ bool tuning_ok(rsc_ctx* ctx, const rsc_tuning& t) {
     if ((p ? rhs_smem<float>(d, t.rhs_pairs[p]) : rhs_smem<double>(d, t.rhs_pairs[p])) > 200 * 1024)
       return false;
   }
-  if (t.synth_radii < 1 || t.synth_radii > 4) return false;
+  if (t.synth_radii < 1 || t.synth_radii > radii_limit((const void*)k_synth<double>, round32(d.nlat2)))
+    return false;
   if (t.analysis_tc != 0 && t.analysis_tc != 1) return false;
   if (t.krylov_split != 0 && t.krylov_split != 1) return false;
   if (t.chain_parts < 1 || t.chain_parts > kMaxChainParts) return false;
@@ -2551,24 +2505,23 @@ rsc_status tune_precision(rsc_ctx* ctx, rsc_tuning& t, cudaEvent_t e0, cudaEvent
   CKS(stage_synth<R>(ctx, ctx->rtmp, ctx->FCU));
   CKS(base_grid<R>(ctx));
   auto pa = [&] { return stage_products_analysis<R>(ctx, true); };
+  // analysis: radii per block x latitudes per staged table chunk
   double best = 1e30;
-  if (p == 1) {   // CUDA-core FP32 analysis: radii per block x latitudes per staged table chunk
-    int br = t.analysis_radii[p], bc = t.analysis_chunk[p];
-    const int rmax = radii_limit((const void*)k_analysis<float>, round32(d.L + 1));
-    ctx->anal_tc = 0;
-    for (int r = 1; r <= rmax; r *= 2) {
-      for (int tc : {16, 32, 48, d.nlat2}) {
-        if (tc > d.nlat2 || analysis_smem<float>(d, r, tc) > 200 * 1024) continue;
-        ctx->rt_anal[p] = r;
-        ctx->atc[p] = tc;
-        const double ms = timeit(pa);
-        CKS(st);
-        if (ms < best) { best = ms; br = r; bc = tc; }
-      }
+  int br = t.analysis_radii[p], bc = t.analysis_chunk[p];
+  const int rmax = radii_limit((const void*)k_analysis<R>, round32(d.L + 1));
+  if (p == 1) ctx->anal_tc = 0;
+  for (int r = 1; r <= rmax; r *= 2) {
+    for (int tc : {16, 32, 48, d.nlat2}) {
+      if (tc > d.nlat2 || analysis_smem<R>(d, r, tc) > 200 * 1024) continue;
+      ctx->rt_anal[p] = r;
+      ctx->atc[p] = tc;
+      const double ms = timeit(pa);
+      CKS(st);
+      if (ms < best) { best = ms; br = r; bc = tc; }
     }
-    ctx->rt_anal[p] = t.analysis_radii[p] = br;
-    ctx->atc[p] = t.analysis_chunk[p] = bc;
   }
+  ctx->rt_anal[p] = t.analysis_radii[p] = br;
+  ctx->atc[p] = t.analysis_chunk[p] = bc;
   if (p == 1) {   // tensor-core analysis against the best CUDA-core shape
     ctx->anal_tc = 1;
     const double ms = timeit(pa);
@@ -2591,9 +2544,19 @@ rsc_status tune_precision(rsc_ctx* ctx, rsc_tuning& t, cudaEvent_t e0, cudaEvent
     }
     ctx->synth_pipe = t.synth_pipe = bpipe;
   }
-  if (p == 0) {   // FP64 synthesis: one shape
-    ctx->tune_ms[1] = timeit([&] { return stage_synth<double>(ctx, ctx->rtmp, ctx->FC); });
-    CKS(st);
+  // synthesis (CUDA-core FP64 path): radii per block
+  if (p == 0) {
+    best = 1e30;
+    int bs = t.synth_radii;
+    const int smax = radii_limit((const void*)k_synth<double>, round32(d.nlat2));
+    for (int r = 1; r <= smax; r *= 2) {
+      ctx->rt_synth[0] = r;
+      const double ms = timeit([&] { return stage_synth<double>(ctx, ctx->rtmp, ctx->FC); });
+      CKS(st);
+      if (ms < best) { best = ms; bs = r; }
+    }
+    ctx->rt_synth[0] = t.synth_radii = bs;
+    ctx->tune_ms[1] = best;
   }
   // right-hand side of Jacobian actions (one shape)
   if (p == 1) {
@@ -2835,8 +2798,6 @@ rsc_status rsc_create(const rsc_params* params, void* stream, rsc_ctx** out) {
   if ((st = build_tc_tables(ctx)) != RSC_OK) return fail(st);
   if ((st = build_ta_tables(ctx)) != RSC_OK) return fail(st);
   if ((st = build_par_tables(ctx)) != RSC_OK) return fail(st);
-  if ((st = build_slice_tables<false>(ctx)) != RSC_OK) return fail(st);
-  if ((st = build_slice_tables<true>(ctx)) != RSC_OK) return fail(st);
   if (cudaMalloc((void**)&ctx->d_status, sizeof(int)) != cudaSuccess ||
       cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess) {
     ctx->err = "cudaMalloc of the status word failed";
@@ -2912,7 +2873,7 @@ rsc_status rsc_destroy(rsc_ctx* ctx) {
                   ctx->AR, ctx->rhs, ctx->mid, ctx->xtmp, ctx->vtmp, ctx->rtmp, ctx->ustate, ctx->ref_tmp, ctx->d_Ef[0], ctx->d_Ef[1], ctx->d_Ef[2], ctx->d_Ef[3], ctx->V, ctx->Vs, ctx->partial,
                   ctx->dots, ctx->AR0, ctx->ta_tiles, ctx->ta_off, ctx->cont_hist, ctx->cont_cond, ctx->amax_v, ctx->amax_i, ctx->d_keT, ctx->d_kedT, ctx->d_ker, ctx->d_kew, ctx->d_diag, ctx->d_cr_pairs, ctx->d_E01, ctx->cr_w, ctx->d_cr_rowf, ctx->d_cr_pairf,
                   ctx->par64[0], ctx->par64[1], ctx->par64[2], ctx->par64[3], ctx->par64[4], ctx->par64[5],
-                  ctx->par32[0], ctx->par32[1], ctx->par32[2], ctx->par32[3], ctx->sl[0].tiles, ctx->sl[0].off, ctx->sl[0].ea, ctx->sl[1].tiles, ctx->sl[1].off, ctx->sl[1].ea};
+                  ctx->par32[0], ctx->par32[1], ctx->par32[2], ctx->par32[3]};
   for (void* b : bufs) cudaFree(b);
   for (int q = 0; q < 8; ++q) {
     cudaFree(ctx->leg64.buf[q]);

@@ -157,6 +157,127 @@ __global__ void k_radial(DevGeom g, const double2* __restrict__ x,
 }
 
 // ---------------------------------------------------------------------------
+// a2: Legendre synthesis.  grid = (nm, ceil(Nd / blockDim.y)), block =
+// (>= nlat2, multiple of 32) x RT radii; the RT threads of one latitude read
+// the same table entries, so the table traffic is served from L1.
+// FC[((fld * Nd + i) * (K+1) + a) * nlat + th], fld = ur, ut, up, wr, wt, wp, Tr, Tt, Tp.
+template <typename R>
+__global__ void k_synth(DevGeom g, DevLegendre<R> T, const typename C2<R>::T* __restrict__ SR,
+                        typename C2<R>::T* __restrict__ FC) {
+  grid_begin();
+  using V = typename C2<R>::T;
+  extern __shared__ unsigned char sh_raw[];
+  const int RT = blockDim.y;
+  V* sh = reinterpret_cast<V*>(sh_raw);  // [RT][nl][8]
+  const int a = blockIdx.x;
+  const int m = g.m_of[a];
+  const int p0 = g.pstart[a];
+  const int nl = g.L - m + 1;
+  const int Nd = g.Nd;
+  const int i0 = blockIdx.y * RT;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  for (int idx = tid; idx < RT * nl * 8; idx += blockDim.x * RT) {
+    const int rr = idx / (nl * 8);
+    const int rem = idx - rr * nl * 8;
+    const int q = rem >> 3, c = rem & 7;
+    const int i = i0 + rr;
+    sh[idx] = (i < Nd) ? SR[((long)(p0 + q) * Nd + i) * 8 + c] : mk<R>(0, 0);
+  }
+  const int t = threadIdx.x;
+  const int i = i0 + threadIdx.y;
+  const bool live = t < g.nlat2 && i < Nd;
+  const V* shr = sh + threadIdx.y * nl * 8;
+  const long off = g.leg_off[a];
+  const int n2 = g.nlat2;
+  // table chunks of QC degrees staged in shared memory by the whole block
+  constexpr int QC = 16;
+  R* tab = reinterpret_cast<R*>(sh + RT * nl * 8);   // [QC][3][n2]
+  R sPr[2][3], sPi[2][3];   // P-sums of ur, wr, dT
+  R dRr[2][5], dRi[2][5];   // dP-sums of Su, Tu, Sw, Tw, ST
+  R qRr[2][5], qRi[2][5];   // Ps-sums of Su, Tu, Sw, Tw, ST
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sPr[s][c] = sPi[s][c] = 0;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) dRr[s][c] = dRi[s][c] = qRr[s][c] = qRi[s][c] = 0;
+  }
+  const int nthr = blockDim.x * RT;
+  for (int qc = 0; qc < nl; qc += QC) {
+    const int nq = min(QC, nl - qc);
+    __syncthreads();
+    for (int idx = tid; idx < nq * 3 * n2; idx += nthr) {
+      const int q = idx / (3 * n2);
+      const int rem = idx - q * 3 * n2;
+      const int w = rem / n2, tt = rem - w * n2;
+      const R* src = (w == 0) ? T.P : (w == 1) ? T.dP : T.Ps;
+      tab[idx] = src[off + (long)(qc + q) * n2 + tt];
+    }
+    __syncthreads();
+    if (live) {
+      for (int q0 = 0; q0 < nq; q0 += 2) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int q = q0 + s;   // qc is even, so the parity of q is that of l - m
+          if (q < nq) {
+            const R pv = tab[(q * 3 + 0) * n2 + t];
+            const R dv = tab[(q * 3 + 1) * n2 + t];
+            const R sv = tab[(q * 3 + 2) * n2 + t];
+            const V* c = shr + (qc + q) * 8;
+            sPr[s][0] += pv * c[0].x; sPi[s][0] += pv * c[0].y;
+            sPr[s][1] += pv * c[3].x; sPi[s][1] += pv * c[3].y;
+            sPr[s][2] += pv * c[6].x; sPi[s][2] += pv * c[6].y;
+            const int vi[5] = {1, 2, 4, 5, 7};
+#pragma unroll
+            for (int u = 0; u < 5; ++u) {
+              dRr[s][u] += dv * c[vi[u]].x; dRi[s][u] += dv * c[vi[u]].y;
+              qRr[s][u] += sv * c[vi[u]].x; qRi[s][u] += sv * c[vi[u]].y;
+            }
+          }
+        }
+      }
+    }
+  }
+  if (!live) return;
+  const R mm = (R)m;
+  const int K1 = g.K + 1, nlat = g.nlat;
+#pragma unroll
+  for (int hemi = 0; hemi < 2; ++hemi) {
+    // north: E + O for P-type and dP-type; south: E - O (P-type), -E + O (dP-type)
+    const R sP = hemi ? (R)-1 : (R)1;
+    const R sD = hemi ? (R)-1 : (R)1;
+    const int th = hemi ? (nlat - 1 - t) : t;
+    R Pr[3], Pi[3], Dr[5], Di[5], Sr[5], Si[5];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      Pr[c] = sPr[0][c] + sP * sPr[1][c];
+      Pi[c] = sPi[0][c] + sP * sPi[1][c];
+    }
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+      Dr[u] = sD * dRr[0][u] + dRr[1][u];
+      Di[u] = sD * dRi[0][u] + dRi[1][u];
+      Sr[u] = qRr[0][u] + sP * qRr[1][u];
+      Si[u] = qRi[0][u] + sP * qRi[1][u];
+    }
+    // i m X = (-m X.y, m X.x)
+    V out[9];
+    out[0] = mk<R>(Pr[0], Pi[0]);                                        // u_r
+    out[1] = mk<R>(Dr[0] - mm * Si[1], Di[0] + mm * Sr[1]);               // u_th = dS_u + i m T_u/s
+    out[2] = mk<R>(-mm * Si[0] - Dr[1], mm * Sr[0] - Di[1]);              // u_ph = i m S_u/s - dT_u
+    out[3] = mk<R>(Pr[1], Pi[1]);                                        // omega_r
+    out[4] = mk<R>(Dr[2] - mm * Si[3], Di[2] + mm * Sr[3]);               // omega_th
+    out[5] = mk<R>(-mm * Si[2] - Dr[3], mm * Sr[2] - Di[3]);              // omega_ph
+    out[6] = mk<R>(Pr[2], Pi[2]);                                        // d_r T
+    out[7] = mk<R>(Dr[4], Di[4]);                                        // (1/r) d_th T
+    out[8] = mk<R>(-mm * Si[4], mm * Sr[4]);                              // (1/(r s)) d_ph T
+#pragma unroll
+    for (int fld = 0; fld < 9; ++fld)
+      FC[(((long)fld * Nd + i) * K1 + a) * nlat + th] = out[fld];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // a6: Legendre analysis.  grid = (nm, ceil(Nd / blockDim.y)), block =
 // (>= L + 1, multiple of 32) x RT radii; the Legendre tables are staged TC latitudes at a
 // time (dynamic shared memory RT 8 nlat/2 sizeof(V) + TC 3 (L + 1) sizeof(R)).

@@ -167,3 +167,24 @@ def test_launches_in_a_row_and_one_by_one(torch, L, Ms, Nr, n, precision):
         out.append(U)
     assert torch.equal(out[0], out[1])
     gpu.close()
+
+
+# The FP64 transforms hold every input to its own 53 bits, whatever else stands in its row or column.
+# An action is linear, so scaled by 2^-1035 (every entry subnormal, 39 bits left of an entry of 1) it
+# gives the scaled result.  Rounding to multiples of 2^-1074 at each stage is 2^-39 of 1; fields and
+# intermediates down to 2^-20 of 1 keep 2^-19: bound 2^-19 per field.  A transform that reads
+# subnormals as zero loses the products, which are most of the action of this state.
+@pytest.mark.parametrize("L,Ms,Nr", [(15, 4, 10), (47, 12, 13)])
+def test_action_scaled_into_subnormals(torch, L, Ms, Nr):
+    from paper_2508_16635_gb300 import RotatingShell
+    s = Shell(L, Ms, Nr, 1e-1, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-1, 80.0)
+    x = torch.tensor(s.conductive_state() + si.perturbation(L, Ms, Nr, seed=49, amp=10.0), device="cuda")
+    u = torch.tensor(si.random_vector(L, Ms, Nr, seed=50), device="cuda")
+    want = gpu.apply_jacobian(x, 0.4, -1, u, 200.0).cpu().numpy()
+    linear = gpu.apply_jacobian(torch.zeros_like(x), 0.4, -1, u, 200.0).cpu().numpy()
+    us = torch.tensor(np.ldexp(u.cpu().numpy(), -1035), device="cuda")
+    got = gpu.apply_jacobian(x, 0.4, -1, us, 200.0).cpu().numpy()
+    assert min(_errors(s, linear, want)) > 1e-2          # the products matter in every field
+    assert max(_errors(s, np.ldexp(got, 1035), want)) < 2.0 ** -19
+    gpu.close()
