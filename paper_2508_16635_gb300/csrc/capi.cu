@@ -74,7 +74,9 @@ struct DevFactor {
   float4* Hr = nullptr;
   float4* Wr = nullptr;
   double2 *D64 = nullptr, *G64 = nullptr, *H64 = nullptr, *W64 = nullptr;   // the same in FP64
-  bool cr_no_room = false;   // they did not fit: the FP64 solve runs on the unreduced chains
+  // they did not fit: the FP64 solve runs on the unreduced chains for the life of the slot (a try on
+  // every call would cost a failing factorisation each time); read and set under the share's lock
+  bool cr_no_room = false;
   double cr_s = 0.0;   // wall time of their factorisation (s)
   int cr_on_gpu = 0;   // where it ran
   bool valid = false;
@@ -162,6 +164,8 @@ struct rsc_ctx {
   float4* d_cr_rowf = nullptr;    // [j] {2 / r^3 hi, lo, 2 / r^2 hi, lo}
   float4* d_cr_pairf = nullptr;   // [p][2] {a l, a}, {c (l + 1), c} (coupling coefficients)
   float4* cr_w = nullptr;      // E0 u, E1 u of the odd blocks, [2][2 P Nr]
+  bool cr_ready = false;       // all of these are there
+  bool cr_no_tables = false;   // they did not fit: FP64 solves on the unreduced chains
   // second stream: the temperature solve runs beside the e/f chain solve
   cudaStream_t s2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -241,7 +245,8 @@ template <> const LegDev<float>& leg<float>(const rsc_ctx* ctx) { return ctx->le
     cudaError_t e_ = (call);                                                  \
     if (e_ != cudaSuccess) {                                                  \
       ctx->err = std::string(#call) + ": " + cudaGetErrorString(e_);          \
-      return RSC_ECUDA;                                                       \
+      cudaGetLastError(); /* not left for the check of a later launch */      \
+      return e_ == cudaErrorMemoryAllocation ? RSC_ENOMEM : RSC_ECUDA;        \
     }                                                                         \
   } while (0)
 
@@ -929,6 +934,7 @@ rsc_status gpu_factor_cr(rsc_ctx* ctx, DevFactor* f) {
   for (int q = 0; q < 9; ++q)
     if (cudaMalloc(bufs[q], sizes[q] * sizeof(double2)) != cudaSuccess) {
       release();
+      cudaGetLastError();
       ctx->err = "cudaMalloc of the reduced-chain factorisation scratch failed";
       return RSC_ENOMEM;
     }
@@ -993,7 +999,8 @@ rsc_status gpu_factor_cr(rsc_ctx* ctx, DevFactor* f) {
   ctx->launches += 8;
   if (e != cudaSuccess) {
     ctx->err = std::string("CUDA error in the reduced-chain factorisation: ") + cudaGetErrorString(e);
-    return RSC_ECUDA;
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? RSC_ENOMEM : RSC_ECUDA;
   }
   for (int c = 0; c < nchains; ++c)
     if (hs[c]) {
@@ -1003,51 +1010,73 @@ rsc_status gpu_factor_cr(rsc_ctx* ctx, DevFactor* f) {
   return RSC_OK;
 }
 
-// The reduced-chain tables of the context (pair lists, E0 / E1 as double-float pairs, the
-// w buffer) on first use, and the reduced factors of f if it has none (on the GPU where the
-// FP64 factorisation runs there, else on the host).
+// The reduced-chain tables of the context: pair lists, E0 / E1 as double-float pairs and in FP64, the
+// coupling factors, the w buffer.
+rsc_status upload_cr_tables(rsc_ctx* ctx) {
+  const Dims& d = ctx->d;
+  std::vector<int> pairs;
+  for (int parity = 1; parity >= 0; --parity) {
+    for (int p = 0; p < d.P; ++p)
+      if (((ctx->t.pair_l[p] - ctx->t.pair_m[p]) & 1) == parity) pairs.push_back(p);
+    if (parity == 1) ctx->n_cr_odd = (int)pairs.size();
+  }
+  ctx->n_cr_even = (int)pairs.size() - ctx->n_cr_odd;
+  CKS(upload(ctx, &ctx->d_cr_pairs, pairs.data(), pairs.size()));
+  std::vector<float2> e(2 * (size_t)d.Nr * d.Nr);
+  for (size_t i = 0; i < e.size(); ++i) {
+    const size_t nn = (size_t)d.Nr * d.Nr;
+    const double a = i < nn ? ctx->t.Ec[0][i] : ctx->t.Ec[1][i - nn];
+    const float ah = (float)a;
+    e[i] = make_float2(ah, (float)(a - (double)ah));
+  }
+  CKS(upload(ctx, &ctx->d_E01, e.data(), e.size()));
+  std::vector<double2> e64((size_t)d.Nr * d.Nr);
+  for (size_t i = 0; i < e64.size(); ++i) e64[i] = make_double2(ctx->t.Ec[0][i], ctx->t.Ec[1][i]);
+  CKS(upload(ctx, &ctx->d_E01_64, e64.data(), e64.size()));
+  auto pair_of = [](double a, double b) {
+    const float ah = (float)a, bh = (float)b;
+    return make_float4(ah, (float)(a - (double)ah), bh, (float)(b - (double)bh));
+  };
+  std::vector<float4> rowf(d.Nr), pairf(2 * (size_t)d.P);
+  for (int j = 0; j < d.Nr; ++j) {
+    const double r = ctx->t.rc[j], sc = 2.0 / (r * r);
+    rowf[j] = pair_of(sc / r, sc);
+  }
+  for (int p = 0; p < d.P; ++p) {
+    double k[2];
+    coupling_factors(ctx->t.pair_l[p], ctx->t.pair_m[p], k);
+    const double l = ctx->t.pair_l[p];
+    pairf[2 * p] = pair_of(k[0] * l, k[0]);
+    pairf[2 * p + 1] = pair_of(k[1] * (l + 1.0), k[1]);
+  }
+  CKS(upload(ctx, &ctx->d_cr_rowf, rowf.data(), rowf.size()));
+  CKS(upload(ctx, &ctx->d_cr_pairf, pairf.data(), pairf.size()));
+  CK(cudaMalloc(&ctx->cr_w, (size_t)2 * 2 * d.P * d.Nr * sizeof(float4)));
+  return RSC_OK;
+}
+
+// They are all there or none is: a solve asks for cr_ready alone.
+rsc_status ensure_cr_tables(rsc_ctx* ctx) {
+  if (ctx->cr_ready) return RSC_OK;
+  const rsc_status st = upload_cr_tables(ctx);
+  if (st == RSC_OK) {
+    ctx->cr_ready = true;
+    return RSC_OK;
+  }
+  void* bufs[] = {ctx->d_cr_pairs, ctx->d_E01, ctx->d_E01_64, ctx->d_cr_rowf, ctx->d_cr_pairf, ctx->cr_w};
+  for (void* b : bufs) cudaFree(b);
+  ctx->d_cr_pairs = nullptr;
+  ctx->d_E01 = nullptr;
+  ctx->d_E01_64 = nullptr;
+  ctx->d_cr_rowf = ctx->d_cr_pairf = ctx->cr_w = nullptr;
+  return st;
+}
+
+// The tables, and the reduced factors of f if it has none (on the GPU where the FP64 factorisation
+// runs there, else on the host).  A shared slot: under the share's lock.
 rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
   const Dims& d = ctx->d;
-  if (!ctx->d_E01) {
-    std::vector<int> pairs;
-    for (int parity = 1; parity >= 0; --parity) {
-      for (int p = 0; p < d.P; ++p)
-        if (((ctx->t.pair_l[p] - ctx->t.pair_m[p]) & 1) == parity) pairs.push_back(p);
-      if (parity == 1) ctx->n_cr_odd = (int)pairs.size();
-    }
-    ctx->n_cr_even = (int)pairs.size() - ctx->n_cr_odd;
-    CKS(upload(ctx, &ctx->d_cr_pairs, pairs.data(), pairs.size()));
-    std::vector<float2> e(2 * (size_t)d.Nr * d.Nr);
-    for (size_t i = 0; i < e.size(); ++i) {
-      const size_t nn = (size_t)d.Nr * d.Nr;
-      const double a = i < nn ? ctx->t.Ec[0][i] : ctx->t.Ec[1][i - nn];
-      const float ah = (float)a;
-      e[i] = make_float2(ah, (float)(a - (double)ah));
-    }
-    CKS(upload(ctx, &ctx->d_E01, e.data(), e.size()));
-    std::vector<double2> e64((size_t)d.Nr * d.Nr);
-    for (size_t i = 0; i < e64.size(); ++i) e64[i] = make_double2(ctx->t.Ec[0][i], ctx->t.Ec[1][i]);
-    CKS(upload(ctx, &ctx->d_E01_64, e64.data(), e64.size()));
-    auto pair_of = [](double a, double b) {
-      const float ah = (float)a, bh = (float)b;
-      return make_float4(ah, (float)(a - (double)ah), bh, (float)(b - (double)bh));
-    };
-    std::vector<float4> rowf(d.Nr), pairf(2 * (size_t)d.P);
-    for (int j = 0; j < d.Nr; ++j) {
-      const double r = ctx->t.rc[j], sc = 2.0 / (r * r);
-      rowf[j] = pair_of(sc / r, sc);
-    }
-    for (int p = 0; p < d.P; ++p) {
-      double k[2];
-      coupling_factors(ctx->t.pair_l[p], ctx->t.pair_m[p], k);
-      const double l = ctx->t.pair_l[p];
-      pairf[2 * p] = pair_of(k[0] * l, k[0]);
-      pairf[2 * p + 1] = pair_of(k[1] * (l + 1.0), k[1]);
-    }
-    CKS(upload(ctx, &ctx->d_cr_rowf, rowf.data(), rowf.size()));
-    CKS(upload(ctx, &ctx->d_cr_pairf, pairf.data(), pairf.size()));
-    CK(cudaMalloc(&ctx->cr_w, (size_t)2 * 2 * d.P * d.Nr * sizeof(float4)));
-  }
+  CKS(ensure_cr_tables(ctx));
   if (f->D64) return RSC_OK;
   const auto t0 = std::chrono::steady_clock::now();
   if (factor_on_device(ctx)) {
@@ -1088,16 +1117,17 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
   return RSC_OK;
 }
 
+std::unique_lock<std::mutex> share_lock(rsc_ctx* ctx) {
+  return ctx->share ? std::unique_lock<std::mutex>(ctx->share->mu) : std::unique_lock<std::mutex>();
+}
+
 rsc_status ensure_cr_locked(rsc_ctx* ctx, DevFactor* f) {
-  if (!ctx->share) return ensure_cr(ctx, f);
-  std::lock_guard<std::mutex> lock(ctx->share->mu);
+  const auto lock = share_lock(ctx);
   return ensure_cr(ctx, f);
 }
 
-// The factors of the unreduced chains, if f has none yet.
+// The factors of the unreduced chains, if f has none yet.  A shared slot: under the share's lock.
 rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
-  std::unique_lock<std::mutex> lock;
-  if (ctx->share) lock = std::unique_lock<std::mutex>(ctx->share->mu);
   if (f->G) return RSC_OK;
   const auto t0 = std::chrono::steady_clock::now();
   const rsc_status st = gpu_factor(ctx, f->dt, *f);
@@ -1106,20 +1136,29 @@ rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
   return st;
 }
 
+rsc_status ensure_full_locked(rsc_ctx* ctx, DevFactor* f) {
+  const auto lock = share_lock(ctx);
+  return ensure_full(ctx, f);
+}
+
 rsc_status get_factor_slot(rsc_ctx* ctx, double dt, DevFactor** out);
 
-// A shared slot gains its reduced factors under the share's lock.
+// A shared slot gains the factors that this context's solves read under the share's lock.
 rsc_status get_factor(rsc_ctx* ctx, double dt, DevFactor** out) {
   CKS(get_factor_slot(ctx, dt, out));
   DevFactor* f = *out;
+  const auto lock = share_lock(ctx);
   if (full_wanted(ctx)) CKS(ensure_full(ctx, f));
-  if (!cr64_wanted(ctx) || (f->cr_no_room && !cr_wanted(ctx))) return RSC_OK;
-  const rsc_status st = ensure_cr_locked(ctx, f);
-  if (st != RSC_ENOMEM || cr_wanted(ctx)) return st;
-  // no room for the reduced factorisation (its scratch takes half as much again as the unreduced
-  // factors): the FP64 solve on the unreduced chains
-  cudaGetLastError();
-  f->cr_no_room = true;
+  if (!cr64_wanted(ctx)) return RSC_OK;
+  if (cr_wanted(ctx)) return ensure_cr(ctx, f);
+  if (!ctx->cr_no_tables && !(f->cr_no_room && !f->D64)) {
+    const rsc_status st = ensure_cr(ctx, f);
+    if (st != RSC_ENOMEM) return st;
+    // no room for the tables, or for the reduced factorisation (its scratch takes half as much again
+    // as the unreduced factors): the FP64 solve on the unreduced chains
+    (ctx->cr_ready ? f->cr_no_room : ctx->cr_no_tables) = true;
+    ctx->err.clear();
+  }
   return ensure_full(ctx, f);
 }
 
@@ -1590,7 +1629,7 @@ void launch_gemv_df(rsc_ctx* ctx, const DevFactor* f, double* out) {
 rsc_status stage_solve(rsc_ctx* ctx, const DevFactor* f, double* out, bool df = false,
                        bool temp = true) {
   df = df && ctx->p.precision == RSC_MIXED && ctx->chain_df != 0;
-  const bool cr = df ? cr_wanted(ctx) : cr64_wanted(ctx) && f->D64;
+  const bool cr = df ? cr_wanted(ctx) : cr64_wanted(ctx) && ctx->cr_ready && f->D64;
   const Dims& d = ctx->d;
   // the temperature solve depends only on the right-hand side: it runs on a second stream
   // beside the e/f chain solve (sequentially while tracing, so that every launch is timed)
@@ -2613,7 +2652,7 @@ rsc_status autotune(rsc_ctx* ctx, rsc_tuning* out) {
       const int saved_cr = ctx->chain_cr;
       for (int cr : {0, 1}) {   // the unreduced chains, then the odd-even reduced ones
         ctx->chain_cr = cr;
-        if (!cr && st == RSC_OK) st = ensure_full(ctx, f);
+        if (!cr && st == RSC_OK) st = ensure_full_locked(ctx, f);
         if (cr && (st != RSC_OK || !cr_wanted(ctx))) break;
         if (cr) st = ensure_cr_locked(ctx, f);
         for (int ns : {2, 4}) {
@@ -3162,7 +3201,7 @@ rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, doub
     }
     return RSC_OK;
   }
-  if (which < 3) CKS(ensure_full(ctx, f));
+  if (which < 3) CKS(ensure_full_locked(ctx, f));
   if (which == 3)
     CK(cudaMemcpyAsync(out_host, f->Tinv + index * blk, blk * sizeof(double),
                        cudaMemcpyDeviceToHost, ctx->s));

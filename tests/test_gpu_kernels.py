@@ -188,3 +188,78 @@ def test_action_scaled_into_subnormals(torch, L, Ms, Nr):
     assert min(_errors(s, linear, want)) > 1e-2          # the products matter in every field
     assert max(_errors(s, np.ldexp(got, 1035), want)) < 2.0 ** -19
     gpu.close()
+
+
+def _leave_free(torch, nbytes):
+    """Device memory held so that about nbytes stay free (1 MB tensors, two to a block of the allocator)."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    held = [torch.empty(torch.cuda.mem_get_info()[0] - nbytes - (64 << 20), dtype=torch.uint8, device="cuda")]
+    while torch.cuda.mem_get_info()[0] >= nbytes + (2 << 20):
+        try:
+            held.append(torch.empty(1 << 20, dtype=torch.uint8, device="cuda"))
+        except torch.cuda.OutOfMemoryError:
+            break
+    return held
+
+
+# No room for the reduced factorisation (441 MB of scratch at this size): the FP64 solve runs on the
+# unreduced chains (294 MB of factors) and says nothing of the failed try.  Both solutions are refined,
+# each within 1e-11 of the oracle's at the sizes of test_chain_residual.
+def test_fp64_solve_without_room_for_the_reduced_factors(torch):
+    from paper_2508_16635_gb300 import RotatingShell
+    L, Ms, Nr = 127, 12, 64
+    s = Shell(L, Ms, Nr, 1e-4, 80.0)
+    roomy, tight = (RotatingShell(L, Ms, Nr, 1e-4, 80.0) for _ in range(2))
+    b = torch.tensor(si.random_vector(L, Ms, Nr, seed=51), device="cuda")
+    want = roomy.implicit_solve(b, 2e-3).cpu().numpy()
+    got = torch.empty_like(b)
+    held = _leave_free(torch, 380 << 20)
+    tight.profile(True)
+    tight.implicit_solve(b, 2e-3, out=got)
+    del held
+    torch.cuda.empty_cache()
+    launches = {k: v["launches"] for k, v in tight.profile_report().items()}
+    tight.profile(False)
+    assert launches["chain_reduced"] == 0 and launches["chain_sweep"] == 4, launches
+    assert tight.lib.rsc_last_error(tight._ctx) == b""
+    assert max(_errors(s, got.cpu().numpy(), want)) < 2e-11
+    assert torch.equal(tight.implicit_solve(b, 2e-3), got)      # the slot keeps its choice
+    roomy.close()
+    tight.close()
+
+
+# No room for a context's own tables of the reduced passes (3 MB) while the slot it shares holds the
+# reduced factors: an error while there is no room for the unreduced factors either, then a solve on
+# those; the other context goes on with the reduced ones.
+def test_shared_factors_without_room_for_the_tables(torch):
+    from paper_2508_16635_gb300 import Batch
+    from paper_2508_16635_gb300.rsc import RscError
+    L, Ms, Nr = 127, 12, 64
+    s = Shell(L, Ms, Nr, 1e-4, 80.0)
+    batch = Batch([dict(L=L, Ms=Ms, Nr=Nr, Ek=1e-4, Ra=ra) for ra in (80.0, 90.0)])
+    a, c = batch.shells
+    b = torch.tensor(si.random_vector(L, Ms, Nr, seed=51), device="cuda")
+    want, got = torch.empty_like(b), torch.empty_like(b)
+    torch.cuda.synchronize()
+    a.implicit_solve(b, 2e-3, out=want)
+    torch.cuda.synchronize()
+    held = _leave_free(torch, 0)
+    for _ in range(2):
+        with pytest.raises(RscError) as e:
+            c.implicit_solve(b, 2e-3, out=got)
+        assert e.value.status == 2                               # RSC_ENOMEM
+    del held
+    torch.cuda.empty_cache()
+    c.implicit_solve(b, 2e-3, out=got)
+    torch.cuda.synchronize()
+    assert max(_errors(s, got.cpu().numpy(), want.cpu().numpy())) < 2e-11
+    again = torch.empty_like(b)
+    torch.cuda.synchronize()
+    a.profile(True)
+    a.implicit_solve(b, 2e-3, out=again)
+    launches = a.profile_report()["chain_reduced"]["launches"]
+    a.profile(False)
+    torch.cuda.synchronize()
+    assert launches == 6 and torch.equal(again, want)
+    batch.close()
