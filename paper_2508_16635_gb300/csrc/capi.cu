@@ -810,20 +810,9 @@ rsc_status gpu_factor_temp(rsc_ctx* ctx, double dt, DevFactor& f) {
   return RSC_OK;
 }
 
-// Factorise dt into f (FP64 factors, their double-float copies on a mixed context, the
-// partitioned extras when chain_parts > 1).
-rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
-  const auto t_fac0 = std::chrono::steady_clock::now();
-  if (factor_on_device(ctx)) {
-    // the unreduced chains' factors only where something solves with them (else on first use)
-    CKS(gpu_factor_temp(ctx, dt, f));
-    if (full_wanted(ctx)) CKS(gpu_factor(ctx, dt, f));
-    ctx->factor_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_fac0).count();
-    ctx->factor_on_gpu = 1;
-    f.dt = dt;
-    f.valid = true;
-    return RSC_OK;
-  }
+// The chain factors of one dt on the host (FP64, their double-float copies on a mixed context, the
+// partitioned extras when chain_parts > 1), and the temperature inverses if f has none.
+rsc_status host_factor(rsc_ctx* ctx, double dt, DevFactor& f) {
   HostFactor hf;
   const int bad = build_factor(ctx->p, ctx->d, ctx->t, dt, hf);
   if (bad) {
@@ -835,7 +824,7 @@ rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
   CKS(upload(ctx, &f.G, reinterpret_cast<const double2*>(hf.G.data()), hf.G.size()));
   CKS(upload(ctx, &f.H, reinterpret_cast<const double2*>(hf.H.data()), hf.H.size()));
   CKS(upload(ctx, &f.W, reinterpret_cast<const double2*>(hf.W.data()), hf.W.size()));
-  CKS(upload(ctx, &f.Tinv, hf.Tinv.data(), hf.Tinv.size()));
+  if (!f.Tinv) CKS(upload(ctx, &f.Tinv, hf.Tinv.data(), hf.Tinv.size()));
   if (ctx->p.precision == RSC_MIXED) {
     // double-float copies for the mixed path (chain_df.cuh): hi = the entry rounded to FP32,
     // lo = the remainder rounded to FP32
@@ -879,13 +868,36 @@ rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
       CKS(split_upload(hf.W, &f.Ws));
     }
   }
+  return RSC_OK;
+}
+
+// The temperature inverses of one dt on the host.
+rsc_status host_factor_temp(rsc_ctx* ctx, double dt, DevFactor& f) {
+  HostFactor hf;
+  if (build_factor_temp(ctx->p, ctx->d, ctx->t, dt, hf)) {
+    ctx->err = "singular temperature block";
+    return RSC_ESINGULAR;
+  }
+  return upload(ctx, &f.Tinv, hf.Tinv.data(), hf.Tinv.size());
+}
+
+// Factorise dt into f: the temperature inverses, and the unreduced chains' factors where something
+// solves with them (else on first use).
+rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
+  const auto t_fac0 = std::chrono::steady_clock::now();
+  const bool dev = factor_on_device(ctx);
+  if (dev) {
+    CKS(gpu_factor_temp(ctx, dt, f));
+    if (full_wanted(ctx)) CKS(gpu_factor(ctx, dt, f));
+  } else {
+    CKS(full_wanted(ctx) ? host_factor(ctx, dt, f) : host_factor_temp(ctx, dt, f));
+  }
   ctx->factor_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_fac0).count();
-  ctx->factor_on_gpu = 0;
+  ctx->factor_on_gpu = dev ? 1 : 0;
   f.dt = dt;
   f.valid = true;
   return RSC_OK;
 }
-
 
 // Double-float copy of complex FP64 blocks: hi = the entry rounded to FP32, lo = the
 // remainder rounded to FP32.
@@ -1130,7 +1142,7 @@ rsc_status ensure_cr_locked(rsc_ctx* ctx, DevFactor* f) {
 rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
   if (f->G) return RSC_OK;
   const auto t0 = std::chrono::steady_clock::now();
-  const rsc_status st = gpu_factor(ctx, f->dt, *f);
+  const rsc_status st = factor_on_device(ctx) ? gpu_factor(ctx, f->dt, *f) : host_factor(ctx, f->dt, *f);
   if (st != RSC_OK) free_unreduced(*f);
   ctx->factor_s += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   return st;

@@ -94,6 +94,8 @@ void build_tables(const rsc_params& p, const Dims& d, HostTables& t);
 // nparts > 1: partitioned chains (parts of at least 8 blocks, at most nparts per chain).
 int build_factor(const rsc_params& p, const Dims& d, const HostTables& t, double dt,
                  HostFactor& f, int nparts = 1);
+// Its temperature inverses alone (f.Tinv).  Returns 0 on success.
+int build_factor_temp(const rsc_params& p, const Dims& d, const HostTables& t, double dt, HostFactor& f);
 // Returns 0 on success, or 1 + chain index of a singular block (implicit Coriolis only).
 int build_factor_cr(const rsc_params& p, const Dims& d, const HostTables& t, double dt,
                     HostFactorCR& f);

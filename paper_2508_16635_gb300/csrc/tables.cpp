@@ -11,6 +11,7 @@
 // Coriolis on the left-hand side), the temperature equation Eq. temp, with
 // boundary rows replacing the rows at the walls (Sec. 3.1).
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <stdexcept>
@@ -548,6 +549,32 @@ static bool partition_extras(const Dims& d, const HostTables& t, const Ops& ops,
   return true;
 }
 
+// Temperature: real inverse per l.
+int build_factor_temp(const rsc_params& p, const Dims& d, const HostTables& t, double dt, HostFactor& f) {
+  const int Nr = d.Nr;
+  const size_t blk = (size_t)Nr * Nr;
+  Ops ops{d, t, p.Ek, p.Pr, std::isfinite(dt) ? 1.0 / dt : 0.0, Nr, p.explicit_coriolis != 0};
+  f.Tinv.assign((size_t)(d.L + 1) * blk, 0.0);
+  std::vector<double> D, I;
+  std::vector<int> piv;
+  std::vector<double> St(Nr);
+  for (int l = 0; l <= d.L; ++l) {
+    ops.temp(l, D);
+    for (int r = 0; r < Nr; ++r) {  // row equilibration, as for the chains
+      double mx = 0.0;
+      for (int k = 0; k < Nr; ++k) mx = std::max(mx, std::fabs(D[(size_t)r * Nr + k]));
+      St[r] = 1.0 / mx;
+      for (int k = 0; k < Nr; ++k) D[(size_t)r * Nr + k] *= St[r];
+    }
+    if (!lu_factor(Nr, D, piv)) return 1;
+    I.assign(blk, 0.0);
+    for (int r = 0; r < Nr; ++r) I[(size_t)r * Nr + r] = St[r];
+    lu_solve(Nr, D, piv, Nr, I);
+    std::copy(I.begin(), I.end(), f.Tinv.begin() + (size_t)l * blk);
+  }
+  return 0;
+}
+
 int build_factor(const rsc_params& p, const Dims& d, const HostTables& t, double dt,
                  HostFactor& f, int nparts) {
   const int Nr = d.Nr;
@@ -718,26 +745,7 @@ int build_factor(const rsc_params& p, const Dims& d, const HostTables& t, double
   for (int c = 0; c < nchains; ++c)
     if (bad[c]) return 1 + c;
   if (nparts > 1 && !partition_extras(d, t, ops, cuts, f)) return 1 + nchains;
-  // Temperature: real inverse per l.
-  f.Tinv.assign((size_t)(d.L + 1) * blk, 0.0);
-  std::vector<double> D, I;
-  std::vector<int> piv;
-  std::vector<double> St(Nr);
-  for (int l = 0; l <= d.L; ++l) {
-    ops.temp(l, D);
-    for (int r = 0; r < Nr; ++r) {  // row equilibration, as for the chains
-      double mx = 0.0;
-      for (int k = 0; k < Nr; ++k) mx = std::max(mx, std::fabs(D[(size_t)r * Nr + k]));
-      St[r] = 1.0 / mx;
-      for (int k = 0; k < Nr; ++k) D[(size_t)r * Nr + k] *= St[r];
-    }
-    if (!lu_factor(Nr, D, piv)) return 1 + nchains;
-    I.assign(blk, 0.0);
-    for (int r = 0; r < Nr; ++r) I[(size_t)r * Nr + r] = St[r];
-    lu_solve(Nr, D, piv, Nr, I);
-    std::copy(I.begin(), I.end(), f.Tinv.begin() + (size_t)l * blk);
-  }
-  return 0;
+  return build_factor_temp(p, d, t, dt, f) ? 1 + nchains : 0;
 }
 
 // One level of odd-even reduction of every e/f chain (HostFactorCR): the inverses of the
@@ -778,6 +786,17 @@ int build_factor_cr(const rsc_params& p, const Dims& d, const HostTables& t, dou
         for (int k = 0; k < Nr; ++k) cr[k] -= a * br[k];
       }
   };
+  // The same for a coupling block Am, which is real.
+  auto sub_prod_real = [&](cplx* Cm, const cplx* Am, const cplx* Bm) {
+    for (int r = 0; r < Nr; ++r)
+      for (int q = 0; q < Nr; ++q) {
+        const double a = Am[(size_t)r * Nr + q].real();
+        if (a == 0.0) continue;
+        const cplx* br = Bm + (size_t)q * Nr;
+        cplx* cr = Cm + (size_t)r * Nr;
+        for (int k = 0; k < Nr; ++k) cr[k] -= a * br[k];
+      }
+  };
   auto row_max = [&](const cplx* Mx, std::vector<double>& S) {
     for (int r = 0; r < Nr; ++r)
       for (int k = 0; k < Nr; ++k) S[r] = std::max(S[r], std::abs(Mx[(size_t)r * Nr + k]));
@@ -786,113 +805,152 @@ int build_factor_cr(const rsc_params& p, const Dims& d, const HostTables& t, dou
     for (int r = 0; r < Nr; ++r)
       for (int k = 0; k < Nr; ++k) Mx[(size_t)r * Nr + k] *= S[r];
   };
-  std::vector<int> bad(nchains, 0);
-  auto work = [&](int c) -> bool {
-    const int a = c / 2, cls = c % 2, m = t.m_of[a];
-    const int nb = d.L - m + 1, nodd = nb / 2, nred = (nb + 1) / 2;
-    auto field_of = [&](int i) { return ((i + cls) % 2 == 0) ? 0 : 1; };
+  // Blocks are the tasks, not chains: a chain of m = 0 is twice as long as the mean one and would end
+  // alone.  Chains are taken nth at a time (their P, Q and reduced blocks are scratch), in three
+  // phases: every odd block; every block of the reduced chains; the two arms of every reduced chain,
+  // each in order, then its middle block.
+  const int nth = std::max(1, (int)std::thread::hardware_concurrency());
+  struct Work {   // of a thread
     std::vector<cplx> D, A, C, tmp;
-    std::vector<double> S(Nr);
+    std::vector<double> S;
     std::vector<int> piv;
-    // odd blocks i = 2q + 1: D_i^-1, Pq = D_i^-1 A_i, Qq = D_i^-1 C_i
-    std::vector<cplx> Pm((size_t)nodd * blk, cplx(0.0)), Qm((size_t)nodd * blk, cplx(0.0));
-    for (int q = 0; q < nodd; ++q) {
-      const int i = 2 * q + 1, l = m + i, fld = field_of(i);
-      ops.diag(fld, l, m, D);
-      std::fill(S.begin(), S.end(), 0.0);
-      row_max(D.data(), S);
-      for (int r = 0; r < Nr; ++r) S[r] = 1.0 / S[r];
-      scale_rows(D.data(), S);
-      if (!lu_factor(Nr, D, piv)) return false;
-      tmp.assign(blk, cplx(0.0));
-      for (int r = 0; r < Nr; ++r) tmp[(size_t)r * Nr + r] = S[r];
-      lu_solve(Nr, D, piv, Nr, tmp);
-      std::copy(tmp.begin(), tmp.end(), &f.Dinv[(f.odd_off[c] + q) * blk]);
-      ops.coupling(fld, l, m, -1, A);
-      scale_rows(A.data(), S);
-      lu_solve(Nr, D, piv, Nr, A);
-      std::copy(A.begin(), A.end(), &Pm[(size_t)q * blk]);
-      if (i + 1 < nb) {
-        ops.coupling(fld, l, m, +1, C);
-        scale_rows(C.data(), S);
-        lu_solve(Nr, D, piv, Nr, C);
-        std::copy(C.begin(), C.end(), &Qm[(size_t)q * blk]);
-      }
-    }
-    // reduced chain on the even blocks j = 2 tt
-    std::vector<cplx> Dr((size_t)nred * blk, cplx(0.0)), Ar((size_t)nred * blk, cplx(0.0)),
-        Cr((size_t)nred * blk, cplx(0.0));
-    for (int tt = 0; tt < nred; ++tt) {
-      const int j = 2 * tt, l = m + j, fld = field_of(j);
-      ops.diag(fld, l, m, D);
-      cplx* dr = &Dr[(size_t)tt * blk];
-      std::copy(D.begin(), D.end(), dr);
-      if (j >= 1) {
-        ops.coupling(fld, l, m, -1, A);
-        sub_prod(dr, A.data(), &Qm[(size_t)(tt - 1) * blk]);
-        if (j >= 2) sub_prod(&Ar[(size_t)tt * blk], A.data(), &Pm[(size_t)(tt - 1) * blk]);
-      }
-      if (j + 1 < nb) {
-        ops.coupling(fld, l, m, +1, C);
-        sub_prod(dr, C.data(), &Pm[(size_t)tt * blk]);
-        if (j + 2 < nb) sub_prod(&Cr[(size_t)tt * blk], C.data(), &Qm[(size_t)tt * blk]);
-      }
-    }
-    // twisted block factors of the reduced chain
-    const int km = (nred - 1) / 2;
-    auto slot = [&](std::vector<cplx>& v, int tt) { return &v[(f.red_off[c] + tt) * blk]; };
-    auto factor_block = [&](int tt, bool up, bool down) -> bool {
-      // up: subtract A' W_{tt-1}; down: subtract C' W_{tt+1}
-      const bool hasA = tt > 0, hasC = tt < nred - 1;
-      std::fill(S.begin(), S.end(), 0.0);
-      row_max(&Dr[(size_t)tt * blk], S);
-      if (hasA) row_max(&Ar[(size_t)tt * blk], S);
-      if (hasC) row_max(&Cr[(size_t)tt * blk], S);
-      for (int r = 0; r < Nr; ++r) S[r] = 1.0 / S[r];
-      D.assign(Dr.begin() + (size_t)tt * blk, Dr.begin() + (size_t)(tt + 1) * blk);
-      if (up) sub_prod(D.data(), &Ar[(size_t)tt * blk], slot(f.W, tt - 1));
-      if (down) sub_prod(D.data(), &Cr[(size_t)tt * blk], slot(f.W, tt + 1));
-      scale_rows(D.data(), S);
-      if (!lu_factor(Nr, D, piv)) return false;
-      tmp.assign(blk, cplx(0.0));
-      for (int r = 0; r < Nr; ++r) tmp[(size_t)r * Nr + r] = S[r];
-      lu_solve(Nr, D, piv, Nr, tmp);
-      std::copy(tmp.begin(), tmp.end(), slot(f.G, tt));
-      // top / middle: H = D'^-1 A', W = D'^-1 C';  bottom: H = E'^-1 C', W = E'^-1 A'
-      const bool bottom = tt > km;
-      const std::vector<cplx>& Hsrc = bottom ? Cr : Ar;
-      const std::vector<cplx>& Wsrc = bottom ? Ar : Cr;
-      const bool hasH = bottom ? hasC : hasA, hasW = bottom ? hasA : hasC;
-      if (hasH) {
-        A.assign(Hsrc.begin() + (size_t)tt * blk, Hsrc.begin() + (size_t)(tt + 1) * blk);
-        scale_rows(A.data(), S);
-        lu_solve(Nr, D, piv, Nr, A);
-        std::copy(A.begin(), A.end(), slot(f.H, tt));
-      }
-      if (hasW) {
-        C.assign(Wsrc.begin() + (size_t)tt * blk, Wsrc.begin() + (size_t)(tt + 1) * blk);
-        scale_rows(C.data(), S);
-        lu_solve(Nr, D, piv, Nr, C);
-        std::copy(C.begin(), C.end(), slot(f.W, tt));
-      }
-      return true;
-    };
-    for (int tt = 0; tt < km; ++tt)
-      if (!factor_block(tt, tt > 0, false)) return false;
-    for (int tt = nred - 1; tt > km; --tt)
-      if (!factor_block(tt, false, tt < nred - 1)) return false;
-    return factor_block(km, km > 0, km < nred - 1);
   };
-  const int nth = std::max(1, std::min<int>(nchains, (int)std::thread::hardware_concurrency()));
-  std::vector<std::thread> pool;
-  for (int w = 0; w < nth; ++w)
-    pool.emplace_back([&, w]() {
-      for (int c = w; c < nchains; c += nth)
-        if (!work(c)) bad[c] = 1;
-    });
-  for (auto& th : pool) th.join();
-  for (int c = 0; c < nchains; ++c)
-    if (bad[c]) return 1 + c;
+  std::vector<Work> ws(nth);
+  for (Work& w : ws) w.S.resize(Nr);
+  struct Chain {
+    int c, m, cls, nb, nodd, nred, km;
+    std::vector<cplx> P, Q, D, A, C;   // D^-1 A, D^-1 C of the odd blocks; the reduced chain
+    std::atomic<int> left{2}, bad{0};
+    int field(int i) const { return ((i + cls) % 2 == 0) ? 0 : 1; }
+  };
+  struct Task { Chain* ch; int i; };
+  auto parallel = [&](const std::vector<Task>& tasks, auto&& fn) {
+    std::atomic<size_t> next{0};
+    std::vector<std::thread> pool;
+    for (int w = 0; w < std::min<int>(nth, (int)tasks.size()); ++w)
+      pool.emplace_back([&, w]() {
+        for (size_t k; (k = next++) < tasks.size();) fn(*tasks[k].ch, tasks[k].i, ws[w]);
+      });
+    for (auto& th : pool) th.join();
+  };
+  // odd block i = 2q + 1: D_i^-1, P_q = D_i^-1 A_i, Q_q = D_i^-1 C_i
+  auto odd_block = [&](Chain& ch, int q, Work& w) {
+    const int i = 2 * q + 1, l = ch.m + i, fld = ch.field(i);
+    ops.diag(fld, l, ch.m, w.D);
+    std::fill(w.S.begin(), w.S.end(), 0.0);
+    row_max(w.D.data(), w.S);
+    for (int r = 0; r < Nr; ++r) w.S[r] = 1.0 / w.S[r];
+    scale_rows(w.D.data(), w.S);
+    if (!lu_factor(Nr, w.D, w.piv)) {
+      ch.bad = 1;
+      return;
+    }
+    w.tmp.assign(blk, cplx(0.0));
+    for (int r = 0; r < Nr; ++r) w.tmp[(size_t)r * Nr + r] = w.S[r];
+    lu_solve(Nr, w.D, w.piv, Nr, w.tmp);
+    std::copy(w.tmp.begin(), w.tmp.end(), &f.Dinv[(f.odd_off[ch.c] + q) * blk]);
+    ops.coupling(fld, l, ch.m, -1, w.A);
+    scale_rows(w.A.data(), w.S);
+    lu_solve(Nr, w.D, w.piv, Nr, w.A);
+    std::copy(w.A.begin(), w.A.end(), &ch.P[(size_t)q * blk]);
+    if (i + 1 < ch.nb) {
+      ops.coupling(fld, l, ch.m, +1, w.C);
+      scale_rows(w.C.data(), w.S);
+      lu_solve(Nr, w.D, w.piv, Nr, w.C);
+      std::copy(w.C.begin(), w.C.end(), &ch.Q[(size_t)q * blk]);
+    }
+  };
+  // block tt of the reduced chain, on the even block j = 2 tt
+  auto reduced_block = [&](Chain& ch, int tt, Work& w) {
+    if (ch.bad) return;
+    const int j = 2 * tt, l = ch.m + j, fld = ch.field(j);
+    ops.diag(fld, l, ch.m, w.D);
+    cplx* dr = &ch.D[(size_t)tt * blk];
+    std::copy(w.D.begin(), w.D.end(), dr);
+    if (j >= 1) {
+      ops.coupling(fld, l, ch.m, -1, w.A);
+      sub_prod_real(dr, w.A.data(), &ch.Q[(size_t)(tt - 1) * blk]);
+      if (j >= 2) sub_prod_real(&ch.A[(size_t)tt * blk], w.A.data(), &ch.P[(size_t)(tt - 1) * blk]);
+    }
+    if (j + 1 < ch.nb) {
+      ops.coupling(fld, l, ch.m, +1, w.C);
+      sub_prod_real(dr, w.C.data(), &ch.P[(size_t)tt * blk]);
+      if (j + 2 < ch.nb) sub_prod_real(&ch.C[(size_t)tt * blk], w.C.data(), &ch.Q[(size_t)tt * blk]);
+    }
+  };
+  // twisted block factors of the reduced chain
+  auto slot = [&](std::vector<cplx>& v, const Chain& ch, int tt) { return &v[(f.red_off[ch.c] + tt) * blk]; };
+  auto factor_block = [&](Chain& ch, int tt, bool up, bool down, Work& w) -> bool {
+    // up: subtract A' W_{tt-1}; down: subtract C' W_{tt+1}
+    const bool hasA = tt > 0, hasC = tt < ch.nred - 1;
+    std::fill(w.S.begin(), w.S.end(), 0.0);
+    row_max(&ch.D[(size_t)tt * blk], w.S);
+    if (hasA) row_max(&ch.A[(size_t)tt * blk], w.S);
+    if (hasC) row_max(&ch.C[(size_t)tt * blk], w.S);
+    for (int r = 0; r < Nr; ++r) w.S[r] = 1.0 / w.S[r];
+    w.D.assign(ch.D.begin() + (size_t)tt * blk, ch.D.begin() + (size_t)(tt + 1) * blk);
+    if (up) sub_prod(w.D.data(), &ch.A[(size_t)tt * blk], slot(f.W, ch, tt - 1));
+    if (down) sub_prod(w.D.data(), &ch.C[(size_t)tt * blk], slot(f.W, ch, tt + 1));
+    scale_rows(w.D.data(), w.S);
+    if (!lu_factor(Nr, w.D, w.piv)) return false;
+    w.tmp.assign(blk, cplx(0.0));
+    for (int r = 0; r < Nr; ++r) w.tmp[(size_t)r * Nr + r] = w.S[r];
+    lu_solve(Nr, w.D, w.piv, Nr, w.tmp);
+    std::copy(w.tmp.begin(), w.tmp.end(), slot(f.G, ch, tt));
+    // top / middle: H = D'^-1 A', W = D'^-1 C';  bottom: H = E'^-1 C', W = E'^-1 A'
+    const bool bottom = tt > ch.km;
+    const std::vector<cplx>& Hsrc = bottom ? ch.C : ch.A;
+    const std::vector<cplx>& Wsrc = bottom ? ch.A : ch.C;
+    const bool hasH = bottom ? hasC : hasA, hasW = bottom ? hasA : hasC;
+    if (hasH) {
+      w.A.assign(Hsrc.begin() + (size_t)tt * blk, Hsrc.begin() + (size_t)(tt + 1) * blk);
+      scale_rows(w.A.data(), w.S);
+      lu_solve(Nr, w.D, w.piv, Nr, w.A);
+      std::copy(w.A.begin(), w.A.end(), slot(f.H, ch, tt));
+    }
+    if (hasW) {
+      w.C.assign(Wsrc.begin() + (size_t)tt * blk, Wsrc.begin() + (size_t)(tt + 1) * blk);
+      scale_rows(w.C.data(), w.S);
+      lu_solve(Nr, w.D, w.piv, Nr, w.C);
+      std::copy(w.C.begin(), w.C.end(), slot(f.W, ch, tt));
+    }
+    return true;
+  };
+  // one arm of a reduced chain (0 above the middle, 1 below); the later one goes on with the middle
+  auto arm = [&](Chain& ch, int below, Work& w) {
+    bool ok = !ch.bad;
+    if (!below)
+      for (int tt = 0; tt < ch.km && ok; ++tt) ok = factor_block(ch, tt, tt > 0, false, w);
+    else
+      for (int tt = ch.nred - 1; tt > ch.km && ok; --tt) ok = factor_block(ch, tt, false, tt < ch.nred - 1, w);
+    if (!ok) ch.bad = 1;
+    if (--ch.left == 0 && !ch.bad && !factor_block(ch, ch.km, ch.km > 0, ch.km < ch.nred - 1, w)) ch.bad = 1;
+  };
+  for (int c0 = 0; c0 < nchains; c0 += nth) {
+    const int n = std::min(nth, nchains - c0);
+    std::vector<Chain> chains(n);
+    std::vector<Task> odd, red, arms;
+    for (int q = 0; q < n; ++q) {
+      Chain& ch = chains[q];
+      ch.c = c0 + q;
+      ch.m = t.m_of[ch.c / 2];
+      ch.cls = ch.c % 2;
+      ch.nb = d.L - ch.m + 1;
+      ch.nodd = ch.nb / 2;
+      ch.nred = (ch.nb + 1) / 2;
+      ch.km = (ch.nred - 1) / 2;
+      for (std::vector<cplx>* v : {&ch.P, &ch.Q}) v->assign((size_t)ch.nodd * blk, cplx(0.0));
+      for (std::vector<cplx>* v : {&ch.D, &ch.A, &ch.C}) v->assign((size_t)ch.nred * blk, cplx(0.0));
+      for (int k = 0; k < ch.nodd; ++k) odd.push_back({&ch, k});
+      for (int k = 0; k < ch.nred; ++k) red.push_back({&ch, k});
+      for (int k = 0; k < 2; ++k) arms.push_back({&ch, k});   // longest chains first
+    }
+    parallel(odd, odd_block);
+    parallel(red, reduced_block);
+    parallel(arms, arm);
+    for (const Chain& ch : chains)
+      if (ch.bad) return 1 + ch.c;
+  }
   return 0;
 }
 

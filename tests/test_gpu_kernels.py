@@ -263,3 +263,30 @@ def test_shared_factors_without_room_for_the_tables(torch):
     torch.cuda.synchronize()
     assert launches == 6 and torch.equal(again, want)
     batch.close()
+
+
+# Only the factors that the solves of a context read are built, on the host (N_r > 96, factor_gpu = 0) as
+# on the device.  A set is the 2 P blocks of N_r x N_r complex numbers, FP64 or double-float: reduced
+# chains D^-1 of half the blocks and G, H, W of the other half (2 sets per precision), unreduced ones
+# 3.  Half a set (20 MB) is left to the tables and to kernels loaded on first use.
+@pytest.mark.parametrize("Nr,precision,tuning,sets", [
+    (97, "fp64", {}, 2), (96, "fp64", {"factor_gpu": 0}, 2), (96, "fp64", {}, 2),
+    (97, "mixed", {}, 4), (96, "mixed", {}, 4)])
+def test_factors_that_nothing_reads_are_not_built(torch, Nr, precision, tuning, sets):
+    from paper_2508_16635_gb300 import RotatingShell
+    L, Ms = 31, 4
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0, precision=precision)
+    gpu.set_tuning(dict(gpu.tuning(), **tuning))
+    U = gpu.conductive_state()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    gpu.step(U, dt=1e-3)
+    torch.cuda.synchronize()
+    one = 2 * gpu.P * Nr * Nr * 16
+    assert free - torch.cuda.mem_get_info()[0] < (sets + 0.5) * one
+    b = torch.tensor(si.random_vector(L, Ms, Nr, seed=53), device="cuda")
+    x = gpu.implicit_solve(b, 1e-3)
+    G = gpu.factor_block(1e-3, "G", 0)          # the unreduced chains', built now
+    assert np.isfinite(G).all() and np.abs(G).max() > 0
+    assert torch.equal(gpu.implicit_solve(b, 1e-3), x)
+    gpu.close()
