@@ -280,8 +280,10 @@ NCU_TRAFFIC_MB = {
 def traffic_variant(name, precision, tuning, dfk):
     """The NCU_TRAFFIC_MB variant of a kernel class under this tuning."""
     if name not in dfk:
-        # FP64 solves run on reduced chains where the chains are whole (no capture of those sweeps)
-        return "fp64_cr" if name == "chain_sweep" and tuning.get("chain_parts") == 1 else "fp64"
+        # FP64 solves run on reduced chains where the chains are whole, on mixed contexts with chain_cr
+        # (no capture of those sweeps)
+        reduced = tuning.get("chain_parts") == 1 and (precision != "mixed" or tuning.get("chain_cr", 0))
+        return "fp64_cr" if name == "chain_sweep" and reduced else "fp64"
     if precision == "mixed" and tuning.get("chain_cr", 0) and name in ("chain_sweep", "chain_reduced"):
         return "df_cr"
     return "df"

@@ -430,7 +430,8 @@ typedef struct {
                               Coriolis only).  Default 1 on a mixed context; 0 = the
                               unreduced chains.  Changes the order of the arithmetic.
                               (FP64 solves run on reduced chains wherever chain_parts = 1,
-                              the Coriolis term is implicit and their factors fit.)     */
+                              the Coriolis term is implicit and their factors fit; on a
+                              mixed context, with chain_cr = 1 only.)                   */
   double ms[6];            /* after rsc_autotune: best times (ms) of products +
                               analysis (mixed), FP64 synthesis, RHS (mixed), FP64 chain
                               solve, double-float chain solve (0 if none ran); zero

@@ -715,16 +715,15 @@ bool factor_on_device(const rsc_ctx* ctx) {
 }
 
 // The FP64 solve runs on odd-even reduced chains (chain_cr.cuh): wherever the chains are whole and
-// coupled.
-bool cr64_wanted(const rsc_ctx* ctx) { return ctx->chain_parts == 1 && !ctx->p.explicit_coriolis; }
-// The double-float solve of the mixed path does too (rsc_tuning chain_cr).
-bool cr_wanted(const rsc_ctx* ctx) {
-  return ctx->p.precision == RSC_MIXED && ctx->chain_cr && cr64_wanted(ctx);
+// coupled, on a mixed context with the double-float solve (rsc_tuning chain_cr).
+bool cr64_wanted(const rsc_ctx* ctx) {
+  return ctx->chain_parts == 1 && !ctx->p.explicit_coriolis &&
+         (ctx->p.precision != RSC_MIXED || ctx->chain_cr);
 }
+// The double-float solve of the mixed path does too.
+bool cr_wanted(const rsc_ctx* ctx) { return ctx->p.precision == RSC_MIXED && cr64_wanted(ctx); }
 // The factors of the unreduced chains are needed.
-bool full_wanted(const rsc_ctx* ctx) {
-  return !cr64_wanted(ctx) || (ctx->p.precision == RSC_MIXED && !ctx->chain_cr);
-}
+bool full_wanted(const rsc_ctx* ctx) { return !cr64_wanted(ctx); }
 
 FacGeom fac_geom(const rsc_ctx* ctx, double dt);
 

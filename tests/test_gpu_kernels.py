@@ -271,7 +271,7 @@ def test_shared_factors_without_room_for_the_tables(torch):
 # 3.  Half a set (20 MB) is left to the tables and to kernels loaded on first use.
 @pytest.mark.parametrize("Nr,precision,tuning,sets", [
     (97, "fp64", {}, 2), (96, "fp64", {"factor_gpu": 0}, 2), (96, "fp64", {}, 2),
-    (97, "mixed", {}, 4), (96, "mixed", {}, 4)])
+    (97, "mixed", {}, 4), (96, "mixed", {}, 4), (96, "mixed", {"chain_cr": 0}, 6)])
 def test_factors_that_nothing_reads_are_not_built(torch, Nr, precision, tuning, sets):
     from paper_2508_16635_gb300 import RotatingShell
     L, Ms = 31, 4
