@@ -2608,12 +2608,26 @@ rsc_status tune_precision(rsc_ctx* ctx, rsc_tuning& t, cudaEvent_t e0, cudaEvent
     ctx->rt_synth[0] = t.synth_radii = bs;
     ctx->tune_ms[1] = best;
   }
-  // right-hand side of Jacobian actions (one shape)
-  if (p == 1) {
-    const RhsParams rp = make_rp(ctx, 200.0, 0.0, 1);
-    ctx->tune_ms[2] = timeit([&] { return stage_rhs<R>(ctx, rp, ctx->rtmp, ctx->rtmp, nullptr, ctx->rhs); });
+  // right-hand side (Jacobian-action mode): pairs per block where k_rhs runs, one shape elsewhere
+  const RhsParams rp = make_rp(ctx, 200.0, 0.0, 1);
+  best = 1e30;
+  int bp = t.rhs_pairs[p];
+  const bool shapes = ctx->p.explicit_coriolis || (p == 1 && ctx->rhs_lin_grid == 0);
+  for (int q : {1, 2, 4, 8}) {
+    if (shapes) {
+      if (!threads_fit((const void*)k_rhs<R>, round32(d.Nr) * q) || rhs_smem<R>(d, q) > 200 * 1024) continue;
+      ctx->ppb[p] = q;
+    }
+    const double ms = timeit([&] { return stage_rhs<R>(ctx, rp, ctx->rtmp, ctx->rtmp, nullptr, ctx->rhs); });
     CKS(st);
+    if (ms < best) {
+      best = ms;
+      if (shapes) bp = q;
+    }
+    if (!shapes) break;
   }
+  ctx->ppb[p] = t.rhs_pairs[p] = bp;
+  if (p == 1) ctx->tune_ms[2] = best;
   return RSC_OK;
 }
 

@@ -290,3 +290,14 @@ def test_factors_that_nothing_reads_are_not_built(torch, Nr, precision, tuning, 
     assert np.isfinite(G).all() and np.abs(G).max() > 0
     assert torch.equal(gpu.implicit_solve(b, 1e-3), x)
     gpu.close()
+
+
+# The autotuner times the block shape of the right-hand side where it has one (explicit Coriolis): eight
+# pairs per block, the first choice at this size, take 1.6 times as long as one, two or four.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_autotune_of_the_explicit_right_hand_side(torch, precision):
+    from paper_2508_16635_gb300 import RotatingShell
+    gpu = RotatingShell(31, 4, 24, 1e-3, 80.0, precision=precision, coriolis="explicit")
+    gpu.set_tuning(dict(gpu.tuning(), rhs_pairs=[8, 8]))
+    assert 8 not in list(gpu.autotune()["rhs_pairs"])
+    gpu.close()
