@@ -369,8 +369,9 @@ rsc_status rsc_batch_newton_rw(rsc_batch* batch, double* const* U, double* C, co
 /* Launch shapes of the transform, right-hand-side and chain kernels (no
  * counterpart in the paper: GPU tiling).  [2] = [FP64 path, mixed path].     */
 typedef struct {
-  int products_warps[2];   /* warps per block of the DFT + grid products kernel       */
-  int products_lats[2];    /* latitudes per warp of that kernel                       */
+  int products_warps[2];   /* kept (1, 2, 4 or 8) and ignored: the shape of the DFT + grid
+                              products kernel follows from the sizes                  */
+  int products_lats[2];    /* kept (1 to 16, a power of two) and ignored              */
   int analysis_radii[2];   /* radii per block of the Legendre analysis                */
   int analysis_chunk[2];   /* latitudes per staged chunk of the analysis tables       */
   int synth_radii;         /* radii per block of the CUDA-core (FP64) synthesis       */

@@ -173,10 +173,9 @@ struct rsc_ctx {
   bool capturing = false;   // the stream is captured into a graph
   int rt_synth[2] = {1, 1}, rt_anal[2] = {1, 1};  // radii per block, [fp64, fp32]
   int radial_f32_grid = 0, rhs_lin_grid = 0;     // persistent FP32 radial kernels (0: not used)
-  int wpb[2] = {0, 0};     // warps per block of the products kernel (0: largest that fits)
+  int wpb[2] = {8, 8}, lpw[2] = {1, 1};   // rsc_tuning products_warps, products_lats: kept, without effect
   int ppb[2] = {0, 0};     // pairs per block of the right-hand-side kernel (0: 256 / Nr)
   int atc[2] = {16, 16};   // latitudes per staged chunk of the analysis tables
-  int lpw[2] = {1, 1};     // latitudes per warp of the products kernel
   int anal_tc = 0;         // 1: tensor-core Legendre analysis on the mixed path
   float* ta_tiles = nullptr;   // its A tiles (hi | lo per (m, parity, table, chunk))
   long* ta_off = nullptr;
@@ -607,21 +606,23 @@ int radial_fixed(const Dims& d) {
   return (d.Nr == 64 && d.Nd == 96) ? 1 : (d.Nr == 96 && d.Nd == 144) ? 2 : 0;
 }
 
+constexpr int kProdSmem = 200 * 1024;   // dynamic shared memory of k_products
+
 template <typename R, int J>
-rsc_status products_attributes(rsc_ctx* ctx, int bytes) {
+rsc_status products_attributes(rsc_ctx* ctx) {
   const void* fns[] = {
       (const void*)k_products<R, kProdStep, true, J>, (const void*)k_products<R, kProdStep, false, J>,
       (const void*)k_products<R, kProdLin, true, J>, (const void*)k_products<R, kProdLin, false, J>,
       (const void*)k_products<R, kProdBase, true, J>, (const void*)k_products<R, kProdBase, false, J>};
-  for (const void* fn : fns) CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  for (const void* fn : fns) CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kProdSmem));
   return RSC_OK;
 }
 
 rsc_status set_smem_limits(rsc_ctx* ctx) {
   const int big = 200 * 1024;
-  CKS((products_attributes<double, 1>(ctx, big)));
-  CKS((products_attributes<float, 1>(ctx, big)));
-  CKS((products_attributes<float, 2>(ctx, big)));
+  CKS((products_attributes<double, 1>(ctx)));
+  CKS((products_attributes<float, 1>(ctx)));
+  CKS((products_attributes<float, 2>(ctx)));
   CK(cudaFuncSetAttribute(k_radial<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
   {
     // the persistent FP32 radial kernels: one or two blocks per SM with the tables staged
@@ -1274,16 +1275,6 @@ rsc_status stage_synth(rsc_ctx* ctx, const double* x, void* FCout) {
   return RSC_OK;
 }
 
-// Bound on the `products_warps` field of rsc_tuning (the shared memory of `wpb` warps with all
-// twiddles staged); the shape of k_products itself follows from the sizes (prod_shape).
-template <typename R>
-size_t products_smem(const Dims& d, bool lin, int wpb) {
-  using V = typename C2<R>::T;
-  const int K1 = d.K + 1, NF = lin ? 18 : 9;
-  return (size_t)wpb * NF * K1 * sizeof(V) + 4 * (size_t)K1 * d.nphi * sizeof(R) +
-         (size_t)wpb * 4 * (d.nphi + 1) * sizeof(R);
-}
-
 // Shared memory of the Legendre analysis for RT radii per block and TC staged latitudes.
 template <typename R>
 size_t analysis_smem(const Dims& d, int RT, int TC) {
@@ -1301,11 +1292,16 @@ size_t rhs_smem(const Dims& d, int ppb) {
 
 // k_products on the coefficients `fc`, mode kProdStep, kProdLin or kProdBase.
 template <typename R>
-void launch_products(rsc_ctx* ctx, int mode, const ProdShape& ps, const void* fc) {
+rsc_status launch_products(rsc_ctx* ctx, int mode, const ProdShape& ps, const void* fc) {
   using V = typename C2<R>::T;
   const Dims& d = ctx->d;
   const DevGeom g = ctx->geom();
   const DevLegendre<R> T = leg<R>(ctx).view();
+  if (ps.smem > (size_t)kProdSmem) {
+    ctx->err = "too many wavenumbers for the grid products: L / Ms = " + std::to_string(d.K) + " takes " +
+               std::to_string(ps.smem) + " bytes of shared memory, " + std::to_string(kProdSmem) + " fit";
+    return RSC_ECUDA;
+  }
   const dim3 grid(d.Nd, (d.nlat + ps.LT - 1) / ps.LT);
   const V* c = reinterpret_cast<const V*>(fc);
   V* fa = reinterpret_cast<V*>(ctx->FA);
@@ -1324,6 +1320,8 @@ void launch_products(rsc_ctx* ctx, int mode, const ProdShape& ps, const void* fc
   using two = std::integral_constant<int, sizeof(R) == 4 ? 2 : 1>;
   if (d.nphi % 2 == 0) ps.J == 2 ? pick(std::true_type{}, two{}) : pick(std::true_type{}, one{});
   else ps.J == 2 ? pick(std::false_type{}, two{}) : pick(std::false_type{}, one{});
+  CK(cudaGetLastError());
+  return RSC_OK;
 }
 
 template <typename R>
@@ -1341,8 +1339,7 @@ rsc_status stage_products_analysis(rsc_ctx* ctx, bool lin) {
   KSpan sp(ctx, RSC_K_PRODUCTS,
            13.0 * d.Nd * K1 * d.nlat * sizeof(V) + (lin ? 9.0 * npts * sizeof(R) : 0.0),
            npts * (36.0 * d.K + (lin ? 60.0 : 30.0) + 16.0 * K1));
-  launch_products<R>(ctx, lin ? kProdLin : kProdStep, ps, ctx->FC);
-  CK(cudaGetLastError());
+  CKS(launch_products<R>(ctx, lin ? kProdLin : kProdStep, ps, ctx->FC));
   }
   {
   KSpan sp(ctx, RSC_K_ANALYSIS,
@@ -2054,9 +2051,7 @@ rsc_status base_grid(rsc_ctx* ctx) {
   KSpan sp(ctx, RSC_K_PRODUCTS,
            9.0 * d.Nd * K1 * d.nlat * sizeof(V) + 9.0 * d.Nd * d.nlat * d.nphi * sizeof(R),
            (double)d.Nd * d.nlat * d.nphi * 36.0 * K1);
-  launch_products<R>(ctx, kProdBase, prod_shape<R>(K1, d.nphi, d.nlat, d.Nd, true), ctx->FCU);
-  CK(cudaGetLastError());
-  return RSC_OK;
+  return launch_products<R>(ctx, kProdBase, prod_shape<R>(K1, d.nphi, d.nlat, d.Nd, true), ctx->FCU);
 }
 
 // Base-state grid coefficients (and grid values) for Jacobian actions.
@@ -2439,9 +2434,6 @@ bool tuning_ok(rsc_ctx* ctx, const rsc_tuning& t) {
   auto pow2 = [](int v, int hi) { return v >= 1 && v <= hi && (v & (v - 1)) == 0; };
   for (int p = 0; p < 2; ++p) {
     if (!pow2(t.products_warps[p], 8)) return false;
-    const size_t sm = p ? products_smem<float>(d, true, t.products_warps[p])
-                        : products_smem<double>(d, true, t.products_warps[p]);
-    if (sm > 190 * 1024) return false;
     const int ra = radii_limit(p ? (const void*)k_analysis<float> : (const void*)k_analysis<double>,
                                round32(d.L + 1));
     if (t.analysis_radii[p] < 1 || t.analysis_radii[p] > ra) return false;
@@ -2474,11 +2466,7 @@ bool tuning_ok(rsc_ctx* ctx, const rsc_tuning& t) {
 void get_tuning(const rsc_ctx* ctx, rsc_tuning* t) {
   const Dims& d = ctx->d;
   for (int p = 0; p < 2; ++p) {
-    int w = ctx->wpb[p] > 0 ? ctx->wpb[p] : 8;
-    while (w > 1 && (p ? products_smem<float>(d, true, w) : products_smem<double>(d, true, w)) >
-                        190 * 1024)
-      w /= 2;
-    t->products_warps[p] = w;
+    t->products_warps[p] = ctx->wpb[p];
     t->analysis_radii[p] = ctx->rt_anal[p];
     t->rhs_pairs[p] = ctx->ppb[p] > 0 ? ctx->ppb[p] : std::max(1, 256 / round32(d.Nr));
     t->analysis_chunk[p] = ctx->atc[p];

@@ -301,3 +301,34 @@ def test_autotune_of_the_explicit_right_hand_side(torch, precision):
     gpu.set_tuning(dict(gpu.tuning(), rhs_pairs=[8, 8]))
     assert 8 not in list(gpu.autotune()["rhs_pairs"])
     gpu.close()
+
+
+# Many wavenumbers: 48 and 64 (the shapes of a tuning go back in as they came out, in a batch too), 72, the
+# most that the FP64 products hold; 74 is refused in words.  Bounds as test_products_longitude_counts.
+@pytest.mark.parametrize("K,precision", [(47, "fp64"), (63, "fp64"), (63, "mixed"), (71, "fp64")])
+def test_many_wavenumbers(torch, K, precision):
+    from paper_2508_16635_gb300 import Batch, RotatingShell
+    s = Shell(K, 1, 6, 1e-3, 80.0)
+    gpu = RotatingShell(K, 1, 6, 1e-3, 80.0, precision=precision)
+    gpu.set_tuning(gpu.tuning())
+    x = s.conductive_state() + si.perturbation(K, 1, 6, seed=55, amp=3e-2)
+    got = gpu.explicit_terms(torch.tensor(x, device="cuda")).cpu().numpy()
+    want = s.to_real(s.explicit_terms(s.to_complex(x)))
+    assert max(_errors(s, got, want)) < (1e-12 if precision == "fp64" else 2e-5)
+    gpu.close()
+    if K == 47:
+        batch = Batch([dict(L=K, Ms=1, Nr=6, Ek=1e-3, Ra=ra) for ra in (80.0, 90.0)])
+        batch.autotune()
+        batch.close()
+
+
+def test_too_many_wavenumbers_for_the_products(torch):
+    from paper_2508_16635_gb300 import RotatingShell
+    from paper_2508_16635_gb300.rsc import RscError
+    gpu = RotatingShell(73, 1, 6, 1e-3, 80.0)
+    U = gpu.conductive_state()
+    with pytest.raises(RscError, match="too many wavenumbers"):
+        gpu.explicit_terms(U)
+    b = torch.tensor(si.random_vector(73, 1, 6, seed=57), device="cuda")
+    assert torch.isfinite(gpu.implicit_solve(b, 1e-3)).all()      # what needs no products runs
+    gpu.close()
