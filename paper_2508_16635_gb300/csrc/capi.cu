@@ -77,8 +77,8 @@ struct DevFactor {
   // they did not fit: the FP64 solve runs on the unreduced chains for the life of the slot (a try on
   // every call would cost a failing factorisation each time); read and set under the share's lock
   bool cr_no_room = false;
-  double cr_s = 0.0;   // wall time of their factorisation (s)
-  int cr_on_gpu = 0;   // where it ran
+  double cr_s = 0.0;    // wall time of their factorisation (s)
+  double fac_s = 0.0;   // of the temperature operators and the unreduced chains
   bool valid = false;
 };
 
@@ -881,6 +881,11 @@ rsc_status host_factor_temp(rsc_ctx* ctx, double dt, DevFactor& f) {
   return upload(ctx, &f.Tinv, hf.Tinv.data(), hf.Tinv.size());
 }
 
+// The context's last factorisation (rsc_factor_time): every part of f but the double-float solve's own.
+void note_factor(rsc_ctx* ctx, const DevFactor& f) {
+  ctx->factor_s = f.fac_s + (ctx->p.precision == RSC_MIXED ? 0.0 : f.cr_s);
+}
+
 // Factorise dt into f: the temperature inverses, and the unreduced chains' factors where something
 // solves with them (else on first use).
 rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
@@ -892,7 +897,8 @@ rsc_status build_factor_into(rsc_ctx* ctx, double dt, DevFactor& f) {
   } else {
     CKS(full_wanted(ctx) ? host_factor(ctx, dt, f) : host_factor_temp(ctx, dt, f));
   }
-  ctx->factor_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_fac0).count();
+  f.fac_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_fac0).count();
+  note_factor(ctx, f);
   ctx->factor_on_gpu = dev ? 1 : 0;
   f.dt = dt;
   f.valid = true;
@@ -1098,8 +1104,8 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
       return st;
     }
     f->cr_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    f->cr_on_gpu = 1;
     ctx->factor_cr_s = f->cr_s;
+    note_factor(ctx, *f);
     ctx->factor_cr_on_gpu = 1;
     return RSC_OK;
   }
@@ -1123,8 +1129,8 @@ rsc_status ensure_cr(rsc_ctx* ctx, DevFactor* f) {
     return st;
   }
   f->cr_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  f->cr_on_gpu = 0;
   ctx->factor_cr_s = f->cr_s;
+  note_factor(ctx, *f);
   ctx->factor_cr_on_gpu = 0;
   return RSC_OK;
 }
@@ -1144,7 +1150,8 @@ rsc_status ensure_full(rsc_ctx* ctx, DevFactor* f) {
   const auto t0 = std::chrono::steady_clock::now();
   const rsc_status st = factor_on_device(ctx) ? gpu_factor(ctx, f->dt, *f) : host_factor(ctx, f->dt, *f);
   if (st != RSC_OK) free_unreduced(*f);
-  ctx->factor_s += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+  f->fac_s += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+  note_factor(ctx, *f);
   return st;
 }
 
@@ -3229,7 +3236,7 @@ rsc_status rsc_factor_block(rsc_ctx* ctx, double dt, int which, long index, doub
 
 rsc_status rsc_factor_time(const rsc_ctx* ctx, double* seconds, int* on_gpu) {
   if (!ctx) return RSC_EINVAL;
-  if (seconds) *seconds = ctx->factor_s + (ctx->p.precision == RSC_MIXED ? 0.0 : ctx->factor_cr_s);
+  if (seconds) *seconds = ctx->factor_s;
   if (on_gpu) *on_gpu = ctx->factor_on_gpu;
   return RSC_OK;
 }

@@ -332,3 +332,22 @@ def test_too_many_wavenumbers_for_the_products(torch):
     b = torch.tensor(si.random_vector(73, 1, 6, seed=57), device="cuda")
     assert torch.isfinite(gpu.implicit_solve(b, 1e-3)).all()      # what needs no products runs
     gpu.close()
+
+
+def test_factor_time_is_that_of_the_last_factorisation(torch):
+    """Each dt's own parts: the unreduced chains added to one dt do not count for the other."""
+    import time
+    from paper_2508_16635_gb300 import RotatingShell
+    gpu = RotatingShell(31, 4, 64, 1e-3, 80.0)
+    gpu.set_tuning(dict(gpu.tuning(), factor_gpu=0))
+    b = torch.tensor(si.random_vector(31, 4, 64, seed=59), device="cuda")
+    t = {}
+    for dt in (1e-3, 2e-3):
+        gpu.implicit_solve(b, dt)
+        t[dt] = gpu.factor_time()[0]
+    for dt in (1e-3, 2e-3):
+        t0 = time.perf_counter()
+        gpu.factor_block(dt, "G", 0)
+        wall = time.perf_counter() - t0
+        assert t[dt] < gpu.factor_time()[0] <= t[dt] + wall
+    gpu.close()
