@@ -154,6 +154,7 @@ struct rsc_ctx {
   int cluster_df = 8;     // CTAs per cluster of the double-float sweeps
   int chain_parts = 1;    // parts per chain of the double-float solve (1: unpartitioned)
   int nsm = 1;            // SMs of the device
+  int cr_occ[3][2] = {};  // resident CTAs per SM of the reduced passes (double-float), by CTAS 4 and 5
   int chain_cr = 0;       // 1: the double-float solve on odd-even reduced chains (chain_cr.cuh)
   int* d_cr_pairs = nullptr;   // pairs with odd l - m (n_cr_odd), then even (n_cr_even)
   int n_cr_odd = 0, n_cr_even = 0;
@@ -618,8 +619,28 @@ rsc_status products_attributes(rsc_ctx* ctx) {
   return RSC_OK;
 }
 
+// Block of the reduced passes: four lanes per row, the rows in equal passes of at most 64; shared memory of
+// pass 0, 1, 2 (double-float).
+int cr_threads(const Dims& d) {
+  const int np = (d.Nr + 63) / 64;
+  return round32(4 * ((d.Nr + np - 1) / np));
+}
+size_t cr_smem(const Dims& d, int pass) { return (pass == 2 ? 5 : 2) * (size_t)d.Nr * sizeof(float4); }
+
+template <int CTAS>
+rsc_status cr_occupancy(rsc_ctx* ctx, int col) {
+  const void* fns[3] = {(const void*)k_cr_odd_df<CTAS>, (const void*)k_cr_even_df<CTAS>,
+                        (const void*)k_cr_back_df<CTAS>};
+  for (int pass = 0; pass < 3; ++pass)
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->cr_occ[pass][col], fns[pass], cr_threads(ctx->d),
+                                                     cr_smem(ctx->d, pass)));
+  return RSC_OK;
+}
+
 rsc_status set_smem_limits(rsc_ctx* ctx) {
   const int big = 200 * 1024;
+  CKS(cr_occupancy<4>(ctx, 0));
+  CKS(cr_occupancy<5>(ctx, 1));
   CKS((products_attributes<double, 1>(ctx)));
   CKS((products_attributes<float, 1>(ctx)));
   CKS((products_attributes<float, 2>(ctx)));
@@ -1574,21 +1595,20 @@ cudaError_t launch_chain_df(rsc_ctx* ctx, const DevFactor* f, double* out, bool 
 template <int CTAS>
 void launch_cr_pass_df(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) {
   const Dims& d = ctx->d;
-  const size_t v = (size_t)d.Nr * sizeof(float4);
+  const int thr = cr_threads(d);
+  const size_t sm = cr_smem(d, pass);
   const int* odd = ctx->d_cr_pairs;
   const int* even = ctx->d_cr_pairs + ctx->n_cr_odd;
   double2* o = reinterpret_cast<double2*>(out);
-  // four lanes per row, the rows in equal passes of at most 64
-  const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));
   if (pass == 0)
-    launch(ctx, k_cr_odd_df<CTAS>, 2 * ctx->n_cr_odd, thr, 2 * v,
+    launch(ctx, k_cr_odd_df<CTAS>, 2 * ctx->n_cr_odd, thr, sm,
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->rhs, ctx->cr_w);
   else if (pass == 1)
-    launch(ctx, k_cr_even_df<CTAS>, 2 * ctx->n_cr_even, thr, 2 * v,
+    launch(ctx, k_cr_even_df<CTAS>, 2 * ctx->n_cr_even, thr, sm,
         ctx->geom(), even, f->cr_red_off, f->Gr, ctx->d_cr_rowf, ctx->d_cr_pairf, ctx->rhs,
         ctx->cr_w, o);
   else
-    launch(ctx, k_cr_back_df<CTAS>, 2 * ctx->n_cr_odd, thr, 5 * v,
+    launch(ctx, k_cr_back_df<CTAS>, 2 * ctx->n_cr_odd, thr, sm,
         ctx->geom(), odd, f->cr_odd_off, f->Ds, ctx->d_E01, ctx->d_cr_rowf, ctx->d_cr_pairf,
         ctx->rhs, o);
 }
@@ -1599,7 +1619,7 @@ void launch_cr_pass_64(rsc_ctx* ctx, const DevFactor* f, double* out, int pass) 
   const int* odd = ctx->d_cr_pairs;
   const int* even = ctx->d_cr_pairs + ctx->n_cr_odd;
   double2 *o = reinterpret_cast<double2*>(out), *w = reinterpret_cast<double2*>(ctx->cr_w);
-  const int np = (d.Nr + 63) / 64, thr = round32(4 * ((d.Nr + np - 1) / np));   // as launch_cr_pass_df
+  const int thr = cr_threads(d);
   if (pass == 0)
     launch(ctx, k_cr_odd, 2 * ctx->n_cr_odd, thr, 2 * v, ctx->geom(), odd, f->cr_odd_off, f->D64,
                                                         ctx->d_E01_64, ctx->rhs, w);
@@ -1619,8 +1639,9 @@ void launch_cr_pass(rsc_ctx* ctx, const DevFactor* f, double* out, int pass, boo
     launch_cr_pass_64(ctx, f, out, pass);
     return;
   }
-  // five CTAs per SM where all are resident at once that way only (chain_cr.cuh)
-  if (n > 4 * ctx->nsm && n <= 5 * ctx->nsm)
+  // fewer registers where all CTAs are resident at once that way only (chain_cr.cuh)
+  const int* occ = ctx->cr_occ[pass];
+  if (n > occ[0] * ctx->nsm && n <= occ[1] * ctx->nsm)
     launch_cr_pass_df<5>(ctx, f, out, pass);
   else
     launch_cr_pass_df<4>(ctx, f, out, pass);

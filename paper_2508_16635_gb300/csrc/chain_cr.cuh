@@ -27,9 +27,13 @@
 // Measured (one GB300, mean of the three passes, us; eight lanes per row, every row of the tables,
 // predicated columns -> this): 27.7 -> 22.4 at L = 127, 185 -> 163 at L = 255, 13.7 -> 11.1 at
 // L = 52, N_r = 60; 32 % fewer instructions.
-// CTAS, the CTAs per SM that the registers allow, is 4 (64 registers: 163 us at L = 255, where 5
-// with 48 registers took 191), and 5 where that puts all of a launch on the device at once and 4
-// does not (22.4 us at L = 127 against 25.3).
+// CTAS, the CTAs of 256 threads per SM that the registers allow, is 4 (64 registers: 163 us at L = 255,
+// where 5 with 48 registers took 191), and 5 where its occupancy at the launch's own block puts all CTAs on
+// the device at once and that of 4 does not: blocks of 256 threads from 609 to 760 CTAs on 152 SMs, of 192
+// threads from 761 to 1064, of 160 threads from 913 to 1216.  Mean of the passes, 4 / 5, us: inside,
+// N_r = 64 25.1 / 23.3 (704 CTAs), 128 69.9 / 63.2 (704), 48 20.1 / 18.8 (781), 96 53.7 / 48.8 (900),
+// 80 48.4 / 44.1 (1204); outside, N_r = 48 16.1 / 17.8, 80 28.6 / 35.0, 96 36.8 / 43.9 (704),
+// 64 28.5 / 29.4 (900).
 #pragma once
 
 #include "chain_df.cuh"

@@ -351,3 +351,10 @@ def test_factor_time_is_that_of_the_last_factorisation(torch):
         wall = time.perf_counter() - t0
         assert t[dt] < gpu.factor_time()[0] <= t[dt] + wall
     gpu.close()
+
+
+# The build of the passes with fewer registers runs where it alone puts all CTAs on the device at once: 630
+# CTAs of 256 threads (four or five per SM of 152).
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_reduced_chain_passes_in_one_wave(torch, precision):
+    test_reduced_chain_passes(torch, 34, 1, 64, precision)
