@@ -7,8 +7,9 @@
 // of a pair j, N_r - 1 - j from one pair of table sums, and factors, never divisions, in the rows.
 // Measured (one GB300): mean of the three passes 41 us at L = 127, M_s = 12, N_r = 64 (the FP64 pipe 82 %
 // active), 377 us at L = 255, M_s = 8, N_r = 96; a sweep over every second block 63 us (115 over
-// all, L = 127).  Unreduced -> reduced chains: two FP64 steps at L = 127 2251 -> 2008 us, one at L = 255
-// 10110 -> 9704 us, a refined solve at L = 45, M_s = 5, N_r = 37 295 -> 231 us.
+// all, L = 127).  Unreduced -> reduced chains: two FP64 steps at L = 127 3851 -> 3638 us, one at L = 255
+// 20186 -> 19738, ten monitored ones at L = 31 2548 -> 2280, a refined solve at L = 45, M_s = 5, N_r = 37
+// 270 -> 196 us.
 // Grid of each kernel: 2 CTAs (e and f block) per pair (m, l) of the given parity of l - m, 256 threads.
 #pragma once
 

@@ -26,10 +26,11 @@ namespace rsc {
 // since their factorisation, may be (their blocks are on the way to L2 by then).
 // A step is a chain of dependent kernels, 5 to 40 us each at L = 127, and between the last CTA of
 // one and the first load of the next the device did nothing.  Measured (one GB300): steps at
-// L = 7 76 -> 57 us, ten monitored FP64 steps at L = 31 2438 -> 2033, four second-order steps at L = 52
-// 1270 -> 1094, ten mixed steps at L = 127 2650 -> 2462, two FP64 2003 -> 1947, L = 255 7863 -> 7785 us.
+// L = 7 74 -> 51 us, ten monitored FP64 steps at L = 31 2718 -> 2338, four second-order steps at L = 52
+// 1270 -> 1098, ten mixed steps at L = 127 2651 -> 2491, two FP64 3666 -> 3591, four mixed ones at L = 255
+// 7867 -> 7798 us.
 // A kernel does not release the next one early: its CTAs then took the free slots of whichever SMs
-// had any, and one-wave kernels ran unevenly (L = 127 mixed 2730, FP64 2226 us).
+// had any, and one-wave kernels ran unevenly (ten mixed steps at L = 127 2730 us).
 __device__ __forceinline__ void grid_begin() {
   cudaGridDependencySynchronize();
 }

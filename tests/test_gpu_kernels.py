@@ -358,3 +358,21 @@ def test_factor_time_is_that_of_the_last_factorisation(torch):
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_reduced_chain_passes_in_one_wave(torch, precision):
     test_reduced_chain_passes(torch, 34, 1, 64, precision)
+
+
+# Without refinement the FP64 solve on reduced chains holds the bounds of the double-float one, which is not
+# refined either and has the same passes in fewer bits (test_reduced_chain_passes).
+@pytest.mark.parametrize("L,Ms,Nr", [(9, 3, 17), (12, 5, 33), (7, 7, 64)])
+def test_reduced_chain_passes_unrefined(torch, L, Ms, Nr):
+    from paper_2508_16635_gb300 import RotatingShell
+    from tests.test_gpu_parity import U48, _random_rhs, _solve_errors
+    s = Shell(L, Ms, Nr, 1e-3, 80.0)
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0)
+    gpu.set_tuning(dict(gpu.tuning(), refine=0))
+    b = _random_rhs(s, 41)
+    x = gpu.implicit_solve(torch.tensor(s.to_real(b), device="cuda"), 2e-3).cpu().numpy()
+    eta, fwd, fwd_T = _solve_errors(s, 2e-3, b, s.to_complex(x))
+    assert eta < 64 * U48
+    assert fwd < 32 * 1e-10
+    assert fwd_T < 1e-12
+    gpu.close()
