@@ -126,7 +126,6 @@ struct rsc_ctx {
   int factor_gpu = 1;          // 1: factorise on the GPU (k_factor_*), 0: on the host
   int refine = 1;              // iterative-refinement steps of every FP64 e/f chain solve
   double* ref_tmp = nullptr;   // correction of a refinement step
-  double2* res_z = nullptr;    // table products of its residual, [7][P][Nr]
   double factor_s = 0.0;       // wall time of the last factorisation (s)
   int factor_on_gpu = 0;       // where the last factorisation ran
   double factor_cr_s = 0.0;    // the same for the last factorisation of the reduced chains
@@ -1182,6 +1181,11 @@ rsc_status ensure_full_locked(rsc_ctx* ctx, DevFactor* f) {
   return ensure_full(ctx, f);
 }
 
+bool has_full(rsc_ctx* ctx, const DevFactor* f) {
+  const auto lock = share_lock(ctx);
+  return f->G != nullptr;
+}
+
 rsc_status get_factor_slot(rsc_ctx* ctx, double dt, DevFactor** out);
 
 // A shared slot gains the factors that this context's solves read under the share's lock.
@@ -1810,11 +1814,13 @@ rsc_status stage_solve_fp64(rsc_ctx* ctx, const DevFactor* f, double* out) {
       const FacGeom fg = fac_geom(ctx, f->dt);
       // the residual r is in place over b: the next one is r less the operator of the last correction
       const double2* xo = reinterpret_cast<const double2*>(it ? ctx->ref_tmp : out);
+      // its table products, [7][P][Nr], in the workspace of the radial values ([P][Nd][8], read by then)
+      double2* z = reinterpret_cast<double2*>(ctx->SR);
       launch(ctx, k_chain_products, (d.P + ppb - 1) / ppb, 4 * tw, 4 * (size_t)ppb * d.Nr * sizeof(double),
-          fg, ctx->d_EcT0, ctx->d_EcT1, ctx->d_EcT2, ctx->d_EcT4, d.P, xo, ctx->res_z, ppb);
+          fg, ctx->d_EcT0, ctx->d_EcT1, ctx->d_EcT2, ctx->d_EcT4, d.P, xo, z, ppb);
       CK(cudaGetLastError());
       launch(ctx, k_chain_residual, (int)(((long)d.P * d.Nr + 127) / 128), 128, 0,
-          fg, ctx->par64[4], ctx->d_rowf64, ctx->d_pairf64, ctx->d_pair_l, ctx->d_pair_m, d.P, ctx->res_z, xo,
+          fg, ctx->par64[4], ctx->d_rowf64, ctx->d_pairf64, ctx->d_pair_l, ctx->d_pair_m, d.P, z, xo,
           ctx->rhs);
       CK(cudaGetLastError());
     }
@@ -2694,18 +2700,32 @@ rsc_status autotune(rsc_ctx* ctx, rsc_tuning* out) {
       const int saved_cr = ctx->chain_cr;
       for (int cr : {0, 1}) {   // the unreduced chains, then the odd-even reduced ones
         ctx->chain_cr = cr;
-        if (!cr && st == RSC_OK) st = ensure_full_locked(ctx, f);
         if (cr && (st != RSC_OK || !cr_wanted(ctx))) break;
         if (cr) st = ensure_cr_locked(ctx, f);
+        // the unreduced factors are built for the trial where the slot has none (the next solve adds
+        // them if they win), and left out where they do not fit beside the reduced ones
+        DevFactor trial;
+        const DevFactor* fc = f;
+        if (!cr && st == RSC_OK && !has_full(ctx, f)) {
+          fc = &trial;
+          trial.dt = f->dt;
+          trial.Tinv = f->Tinv;
+          st = factor_on_device(ctx) ? gpu_factor(ctx, f->dt, trial) : host_factor(ctx, f->dt, trial);
+        }
+        const bool left_out = st == RSC_ENOMEM;
+        if (left_out) {
+          st = RSC_OK;
+          ctx->err.clear();
+        }
         for (int ns : {2, 4}) {
           for (int cs : {16, 8, 4, 2}) {
-            if (st != RSC_OK) break;
+            if (st != RSC_OK || left_out) break;
             if (!chain_df_ok(ctx->d, cs, ns)) continue;
             ctx->chain_df = ns;
             ctx->cluster_df = cs;
-            st = stage_solve(ctx, f, ctx->xtmp, true);
+            st = stage_solve(ctx, fc, ctx->xtmp, true);
             cudaEventRecord(e0, ctx->s);
-            for (int r = 0; r < 3 && st == RSC_OK; ++r) st = stage_solve(ctx, f, ctx->xtmp, true);
+            for (int r = 0; r < 3 && st == RSC_OK; ++r) st = stage_solve(ctx, fc, ctx->xtmp, true);
             cudaEventRecord(e1, ctx->s);
             if (cudaEventSynchronize(e1) != cudaSuccess) st = RSC_ECUDA;
             float ms = 0;
@@ -2718,6 +2738,8 @@ rsc_status autotune(rsc_ctx* ctx, rsc_tuning* out) {
             }
           }
         }
+        trial.Tinv = nullptr;   // the slot's
+        free_factor(trial);
       }
       ctx->chain_cr = saved_cr;
       if (st == RSC_OK) st = check_status(ctx);
@@ -2924,7 +2946,6 @@ rsc_status rsc_create(const rsc_params* params, void* stream, rsc_ctx** out) {
   if ((st = alloc((void**)&ctx->rtmp, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
   if ((st = alloc((void**)&ctx->ustate, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
   if ((st = alloc((void**)&ctx->ref_tmp, (size_t)n * sizeof(double))) != RSC_OK) return fail(st);
-  if ((st = alloc((void**)&ctx->res_z, 7 * (size_t)d.P * d.Nr * c16)) != RSC_OK) return fail(st);
   ctx->nblk_dot = (int)std::max<long>((n + 1023) / 1024, 152L * 8);   // pass-A chunks, pass-B blocks
   if ((st = alloc((void**)&ctx->partial, (size_t)ctx->nblk_dot * (2 * kMaxKrylov + 4) * sizeof(double))) != RSC_OK)
     return fail(st);
@@ -2947,7 +2968,7 @@ rsc_status rsc_destroy(rsc_ctx* ctx) {
   if (ctx->s2) cudaStreamSynchronize(ctx->s2), cudaStreamDestroy(ctx->s2);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_EcT4, ctx->res_z, ctx->d_rowf64, ctx->d_pairf64, ctx->d_E01_64, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
+  void* bufs[] = {(void*)ctx->d_slots, ctx->d_cslot, ctx->jvp_y, ctx->tc_tiles, ctx->tc_off, ctx->tc_kpad, ctx->d_status, ctx->d_EcT1, ctx->d_EcT4, ctx->d_rowf64, ctx->d_pairf64, ctx->d_E01_64, ctx->d_m_of, ctx->d_pstart, ctx->d_pair_l, ctx->d_pair_m, ctx->d_leg_off,
                   ctx->d_rc, ctx->d_rd, ctx->d_EcT0, ctx->d_EcT2, ctx->d_EdT0, ctx->d_EdT1,
                   ctx->d_EdT2, ctx->d_R0T, ctx->d_R1T, ctx->f_EdT0, ctx->f_EdT1,
                   ctx->f_EdT2, ctx->f_R0T, ctx->f_R1T, ctx->f_rd, ctx->f_EcT0, ctx->f_EcT2, ctx->SR, ctx->FC, ctx->FCU, ctx->UG, ctx->FA,

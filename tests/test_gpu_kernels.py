@@ -376,3 +376,20 @@ def test_reduced_chain_passes_unrefined(torch, L, Ms, Nr):
     assert fwd < 32 * 1e-10
     assert fwd_T < 1e-12
     gpu.close()
+
+
+# The unreduced factors that the autotuner tries are given back: 4 sets stay on a mixed context that it
+# leaves on the reduced chains (sets as above), 6 more if the unreduced ones win.
+def test_autotune_gives_back_the_factors_it_tried(torch):
+    from paper_2508_16635_gb300 import RotatingShell
+    L, Ms, Nr = 31, 4, 96
+    gpu = RotatingShell(L, Ms, Nr, 1e-3, 80.0, precision="mixed")
+    U = gpu.conductive_state()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    t = gpu.autotune()
+    gpu.step(U, dt=200.0)
+    torch.cuda.synchronize()
+    one = 2 * gpu.P * Nr * Nr * 16
+    assert free - torch.cuda.mem_get_info()[0] < ((4 if t["chain_cr"] else 10) + 0.5) * one
+    gpu.close()
