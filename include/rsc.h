@@ -57,7 +57,9 @@ typedef enum {
   RSC_ENOCONV = 4,     /* Newton or GMRES reached its iteration cap           */
   RSC_ENAN = 5,        /* a non-finite residual or Krylov norm                */
   RSC_ESINGULAR = 6,   /* zero pivot while factorising the implicit operator  */
-  RSC_ETIMEOUT = 7,    /* a bounded device wait gave up                       */
+  RSC_ETIMEOUT = 7,    /* a bounded device wait gave up (mixed transforms, asynchronous and
+                          double-float sweeps): looked at by rsc_autotune and the Newton calls,
+                          for every launch since the last look                      */
   RSC_ERESOLUTION = 8  /* a continuation stopped on an under-resolved state   */
 } rsc_status;
 

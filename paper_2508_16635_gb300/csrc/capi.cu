@@ -2256,7 +2256,7 @@ rsc_status check_status(rsc_ctx* ctx) {
   int st = 0;
   CK(cudaMemcpy(&st, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st != 0) {
-    ctx->err = "a bounded device wait gave up (tensor-core synthesis)";
+    ctx->err = "a bounded device wait gave up (tensor-core transforms, chain sweeps)";
     cudaMemset(ctx->d_status, 0, sizeof(int));
     return (rsc_status)st;
   }
